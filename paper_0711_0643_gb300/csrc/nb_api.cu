@@ -1360,7 +1360,8 @@ nb_status nb_autotune(nb_ctx *ctx)
             if (share && !mixed_share_fits(ctx->n_tiles)) continue;
             const int64_t I = ctx->cfg.precision == NB_PREC_FP64 ? f64_variant_I(v) : mixed_variant_I(v);
             if (I > 4 * s && v > 0) continue;        // i-blocks mostly empty
-            if (!share && (s + I - 1) / I > 4096 && v != kMixedFallbackId) continue;   // far too many small work items
+            if (!share && (s + I - 1) / I > 4096 && v != (mixed ? kMixedFallbackId : kF64Variants - 1))
+                continue;   // far too many small work items
             const int64_t nib = (s + I - 1) / I;
             const int64_t R = force_grid(ctx);
             // wave-aligned splits (W = nib * S just below k full waves), the default's
@@ -1376,7 +1377,7 @@ nb_status nb_autotune(nb_ctx *ctx)
             }
             if (share) cands.assign(1, 1);   // the resident-share variant has no split factor
             for (int64_t S : cands) {
-                if (S * s * kPartStride > ctx->part_cap) continue;
+                if (mixed && S * s * kPartStride > ctx->part_cap) continue;
                 ForceArgs F = force_args(ctx, v, (int)S);
                 float t3[3] = {0.f, 0.f, 0.f};
                 CK(cudaEventRecord(e0, ctx->stream));

@@ -925,10 +925,40 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
     }
 }
 
-// ------------------------------------------------------------ FP64 kernels
-// The plain FP64 path: same decomposition, double arithmetic throughout and
-// j-data read through the read-only cache (all lanes of a warp read the same
-// j in the i-loop variant, one broadcast transaction).
+// ------------------------------------------------------------- FP64 kernel
+// The plain FP64 path. It is bound by the FP64 pipe: an FP64 warp instruction holds
+// a sub-partition's unit for ~64 clocks here, whatever its active lanes, so what
+// counts is the number of FP64 instructions per pair (32, see pair_f64), every lane
+// holding a pair, and the same number of them on every SM:
+//   * a CTA (8 warps) takes an i-block of TI = 32 / TJ active particles, one per
+//     group of TJ lanes (TJ > 1 where blocks of 32 would leave lanes empty), and the
+//     warps and the lanes of a group take consecutive j; all lanes of a warp with the
+//     same j read it in one broadcast transaction;
+//   * the (i-block, j unit) pairs, 8 TJ j's to a unit, are laid out in one line and
+//     cut into equal runs, one per CTA of the grid. A run may end one i-block and
+//     begin the next; an i-block's partials are added by the CTA that completes it
+//     (arrival ticket), in CTA order: the same bits on every run.
+// Measured (us per call, before: one i-particle per CTA up to s = 64, i-blocks of 256
+// with at most n_tiles / 4 shares of j above, so 16 of 152 SMs at work at N = 16384):
+// N = 16384: s = 1 18.4 -> 12.3, 64 84 -> 74, 256 2278 -> 250 (the pipe's time for its
+// instructions is 213), N 18020 -> 15310; N = 65536, s = 1024 4587 -> 3820.
+
+// (r2)^(-1/2) by a third-order Householder step from an FP32 estimate q0:
+// e = 1 - r2 q0^2 (q0^2 is exact in FP64 and the difference rounds once, |e| < 2^-21),
+// q = q0 + q0 e (1/2 + 3/8 e), truncation below 2^-64 relative, so q is the correctly
+// rounded value to within a few hundredths of an ulp. The conversions to and from
+// FP32 are moves of the bit fields (FP64 conversions share the narrow pipe). Only
+// where r2 is not comfortably a normal FP32 number: the library function.
+__device__ __forceinline__ double rsqrt_f64(double r2)
+{
+    const int hi = __double2hiint(r2);
+    if ((unsigned)(hi - ((1023 - 120) << 20)) >= (unsigned)(240 << 20)) return rsqrt(r2);
+    const float f = __int_as_float(__funnelshift_l(__double2loint(r2), hi - (896 << 20), 3));
+    const int qb = __float_as_int(rsqrtf(f));
+    const double q0 = __hiloint2double((qb >> 3) + (896 << 20), qb << 29);
+    const double e = fma(-r2, q0 * q0, 1.0);
+    return fma(q0 * e, fma(e, 0.375, 0.5), q0);
+}
 
 __device__ __forceinline__ void pair_f64(double xj, double yj, double zj, double mj, double vxj, double vyj,
                                          double vzj, const double *xi, double eps2, double *acc, bool self)
@@ -937,7 +967,8 @@ __device__ __forceinline__ void pair_f64(double xj, double yj, double zj, double
     double wx = vxj - xi[3], wy = vyj - xi[4], wz = vzj - xi[5];
     double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
     double rw = fma(dx, wx, fma(dy, wy, dz * wz));
-    double q = self ? 0.0 : rsqrt(r2);
+    double q = rsqrt_f64(r2);
+    if (self) q = 0.0;
     double q2 = q * q;
     double mq = mj * q;
     double mu = mq * q2;
@@ -951,143 +982,185 @@ __device__ __forceinline__ void pair_f64(double xj, double yj, double zj, double
     acc[5] = fma(mu, fma(-al, dz, wz), acc[5]);
 }
 
-__device__ __forceinline__ void load_i64(const ForceArgs &A, int32_t i, double *xi)
+// 0: one particle per i-block (the lanes of a warp on 32 j's)   1: by the block size
+__host__ __device__ __forceinline__ int f64_I(int v) { return v == 0 ? 1 : 32; }
+
+// Particles per i-block of variant 1 for an active count s on `grid` CTAs: the largest
+// power of two up to 32 that leaves at most 1 lane in 8 without a particle (the
+// pipe's time is paid per warp) and spreads the CTAs over enough i-blocks for each to
+// be summed from about kF64Parts partials (one CTA adds them while the others have
+// nothing left; N = 16384, s = 64: 80, 74, 74, 100 us with 8, 16, 32, no limit).
+// Smaller blocks cost a lane tree of a few FP64 additions per item.
+constexpr int kF64Parts = 16;
+__device__ __forceinline__ int f64_block(int64_t s, int64_t grid)
 {
-    const int64_t np = A.n_tiles * kJT;
-    xi[0] = A.xp[i]; xi[1] = A.xp[np + i]; xi[2] = A.xp[2 * np + i];
-    xi[3] = A.vp[i]; xi[4] = A.vp[np + i]; xi[5] = A.vp[2 * np + i];
+    int I = 32;
+    while (I > 1 && (8 * ((s + I - 1) / I * I - s) > s || I * grid > kF64Parts * s)) I >>= 1;
+    return I;
 }
 
-__device__ void work_f64_stream(const ForceArgs &A, int64_t s, int64_t bx, int by, int S, double (*red)[7])
+struct F64Run {
+    int64_t nib, units, U, G;   // i-blocks, units per i-block, all units, CTAs sharing them
+    int64_t jlo, jhi;           // j range
+    int I, unit, slots;         // particles per i-block, j's per unit, partial slots per particle
+};
+
+// CTA whose run holds unit u (run c: units [floor(U c / G), floor(U (c + 1) / G)))
+__device__ __forceinline__ int64_t f64_owner(const F64Run &R, int64_t u) { return ((u + 1) * R.G - 1) / R.U; }
+
+// The sums of i-block b over this CTA's j in [j0, j1): per-warp partial sums through
+// shared memory, component c summed by warp c over the warps, then over the TJ lanes.
+// Returns (in lanes with tj == 0 of warps 0 .. 6) component `warp` of particle ti.
+template <int TJ>
+__device__ __forceinline__ double f64_item(const ForceArgs &A, int64_t s, int64_t ib0, int64_t j0, int64_t j1,
+                                           double (*sacc)[kThreads])
 {
+    constexpr int W = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t gi = A.idx[bx < s ? bx : s - 1];
-    double xi[6];
-    load_i64(A, gi, xi);
+    const int tj = lane % TJ, ti = lane / TJ;
+    const int32_t gi = A.idx[ib0 + ti < s ? ib0 + ti : s - 1];
     const int64_t np = A.n_tiles * kJT;
-    const int64_t tper = qdiv(A.tile_hi - A.tile_lo + S - 1, S);
-    const int64_t t0 = A.tile_lo + (int64_t)by * tper;
-    const int64_t t1 = t0 + tper < A.tile_hi ? t0 + tper : A.tile_hi;
+    const double xi[6] = {A.xp[gi], A.xp[np + gi], A.xp[2 * np + gi], A.vp[gi], A.vp[np + gi], A.vp[2 * np + gi]};
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int64_t j = t0 * kJT + tid; j < t1 * kJT; j += kThreads)
+#pragma unroll 2
+    for (int64_t j = j0 + warp * TJ + tj; j < j1; j += W * TJ)
         pair_f64(__ldg(A.xp + j), __ldg(A.xp + np + j), __ldg(A.xp + 2 * np + j), __ldg(A.m + j),
                  __ldg(A.vp + j), __ldg(A.vp + np + j), __ldg(A.vp + 2 * np + j), xi, A.eps2, acc, j == gi);
 #pragma unroll
-    for (int c = 0; c < 7; ++c) {
-        double x = acc[c];
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if (lane == 0) red[warp][c] = x;
-    }
+    for (int c = 0; c < 7; ++c) sacc[c][tid] = acc[c];
     __syncthreads();
-    if (tid < 7) {
+    double v = 0.0;
+    if (warp < 7) {
+        v = sacc[warp][lane];
+#pragma unroll
+        for (int w = 1; w < W; ++w) v += sacc[warp][w * 32 + lane];
+#pragma unroll
+        for (int off = TJ / 2; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    }
+    return v;
+}
+
+// Adds the n partials of active particles [ib0, ib0 + cnt) in slot order (D lanes per
+// sum, eight loads in flight each, then a lane tree) and writes the results.
+__device__ void f64_finish(const ForceArgs &A, int64_t ib0, int cnt, int n, int slots)
+{
+    const int D = cnt <= 1 ? 32 : (cnt <= 2 ? 16 : (cnt <= 4 ? 8 : (cnt <= 8 ? 4 : (cnt <= 16 ? 2 : 1))));
+    const int d = threadIdx.x % D, per = kThreads / D;
+    for (int q0 = 0; q0 < cnt * 7; q0 += per) {
+        const int q = q0 + threadIdx.x / D;
+        const int qq = q < cnt * 7 ? q : 0;
+        const int64_t ii = ib0 + qq / 7;
+        const double *src = A.part + ii * slots * kPartStride + qq % 7;
         double x = 0.0;
-        for (int wv = 0; wv < kThreads / 32; ++wv) x += red[wv][tid];
-        if (bx < s) A.part[(bx * S + by) * kPartStride + tid] = x;
-    }
-    __syncthreads();
-}
-
-__device__ void work_f64_iloop(const ForceArgs &A, int64_t s, int64_t bx, int by, int S)
-{
-    const int tid = threadIdx.x;
-    const int64_t ii = bx * kThreads + tid;
-    const int32_t gi = A.idx[ii < s ? ii : s - 1];
-    double xi[6];
-    load_i64(A, gi, xi);
-    const int64_t np = A.n_tiles * kJT;
-    const int64_t tper = qdiv(A.tile_hi - A.tile_lo + S - 1, S);
-    const int64_t t0 = A.tile_lo + (int64_t)by * tper;
-    const int64_t t1 = t0 + tper < A.tile_hi ? t0 + tper : A.tile_hi;
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int64_t j = t0 * kJT; j < t1 * kJT; ++j)
-        pair_f64(__ldg(A.xp + j), __ldg(A.xp + np + j), __ldg(A.xp + 2 * np + j), __ldg(A.m + j),
-                 __ldg(A.vp + j), __ldg(A.vp + np + j), __ldg(A.vp + 2 * np + j), xi, A.eps2, acc, j == gi);
-    if (ii < s) {
-        double *dst = A.part + (ii * S + by) * kPartStride;
-        for (int c = 0; c < 7; ++c) dst[c] = acc[c];
-    }
-}
-
-// FP64 counterpart of finish_item: FP64 sums in split order.
-__device__ void finish_item_f64(const ForceArgs &A, int64_t s, int64_t bx, int S, int64_t I, int *last)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const int t = atomicAdd(&A.tickets[bx], 1);
-        *last = (t == S - 1);
-    }
-    __syncthreads();
-    if (*last) {
-        __threadfence();
-        const int64_t ib0 = bx * I;
-        const int64_t ib1 = ib0 + I < s ? ib0 + I : s;
-        const int64_t cnt = (ib1 - ib0) * 7;
-        for (int64_t q = threadIdx.x; q < cnt; q += kThreads) {
-            const int64_t ii = ib0 + q / 7;
-            const int c = (int)(q % 7);
-            const double *src = A.part + ii * S * kPartStride + c;
-            double x = 0.0;
-            // eight loads in flight, added in split order
-            for (int sp0 = 0; sp0 < S; sp0 += 8) {
-                double v[8];
+        for (int sp0 = d; sp0 < n; sp0 += 8 * D) {
+            double v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = sp0 + u < S ? __ldcg(src + (sp0 + u) * kPartStride) : 0.0;
+            for (int u = 0; u < 8; ++u) v[u] = sp0 + u * D < n ? __ldcg(src + (sp0 + u * D) * kPartStride) : 0.0;
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (sp0 + u < S) x += v[u];
-            }
-            put_final(A, ii, c, x);
+            for (int u = 0; u < 8; ++u)
+                if (sp0 + u * D < n) x += v[u];
         }
-        if (threadIdx.x == 0) A.tickets[bx] = 0;
+        for (int off = D / 2; off >= 1; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        if (d == 0 && q < cnt * 7) put_final(A, ii, qq % 7, x);
     }
-    __syncthreads();
 }
 
-__host__ __device__ __forceinline__ int f64_I(int v) { return v == 0 ? 1 : kThreads; }
-
-__global__ void __launch_bounds__(kThreads) force_f64_kernel(ForceArgs A)
+__global__ void __launch_bounds__(kThreads, 2) force_f64_kernel(ForceArgs A)
 {
-    __shared__ double red[kThreads / 32][7];
+    __shared__ double sacc[7][kThreads];
     __shared__ uint64_t inject_bar;
     __shared__ int last;
+    __shared__ F64Run run;
+    const int tid = threadIdx.x;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t s = launch_s(A);
     if (s <= 0) return;
     copy_list(A, s);
     if (A.inject) {
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             mbar_init(&inject_bar, 1);
             fence_mbar_init();
         }
         __syncthreads();
-        if (!mbar_wait(&inject_bar, 0, A.spin_limit) && threadIdx.x == 0) atomicOr(A.status, kStTimeout);
+        if (!mbar_wait(&inject_bar, 0, A.spin_limit) && tid == 0) atomicOr(A.status, kStTimeout);
         return;
     }
-    int variant, S;
-    if (A.force_variant >= 0) {
-        variant = A.force_variant;
-        S = A.force_split;
-    } else {
-        const int b = bucket_of(s);
-        variant = A.tune->variant[b];
+    if (tid == 0) {
+        int variant, S;
+        if (A.force_variant >= 0) {
+            variant = A.force_variant;
+            S = A.force_split;
+        } else {
+            const int b = bucket_of(s);
+            variant = A.tune->variant[b];
+            if (variant < 0 || variant >= kF64Variants) variant = kF64Variants - 1;
+            S = table_split(A.tune->split[b], b, s, A.n, f64_I(variant));
+        }
         if (variant < 0 || variant >= kF64Variants) variant = kF64Variants - 1;
-        S = table_split(A.tune->split[b], b, s, A.n, f64_I(variant));
+        F64Run R;
+        R.I = variant == 0 ? 1 : f64_block(s, gridDim.x);
+        R.unit = kThreads / R.I;   // one j per lane group and warp
+        R.jlo = A.tile_lo * kJT;
+        R.jhi = A.tile_hi * kJT < A.n ? A.tile_hi * kJT : A.n;
+        R.nib = (s + R.I - 1) / R.I;
+        R.units = (R.jhi - R.jlo + R.unit - 1) / R.unit;
+        R.U = R.nib * R.units;
+        // as many CTAs as the split asks for (S of them to an i-block of f64_I(variant))
+        const int64_t nibt = (s + f64_I(variant) - 1) / f64_I(variant);
+        R.G = nibt * (S < 1 ? 1 : S);
+        if (R.G > gridDim.x) R.G = gridDim.x;
+        if (R.G > R.U) R.G = R.U;
+        // a run is at least floor(U / G) units, so an i-block meets at most
+        // ceil(G / nib) + 1 of them; never more partials than there is room for
+        while (R.G > 1 && s * ((R.G + R.nib - 1) / R.nib + 1) * kPartStride > A.part_cap) R.G = (R.G + 1) / 2;
+        R.slots = (int)((R.G + R.nib - 1) / R.nib + 1);
+        run = R;
+        if (blockIdx.x == 0) *A.split_used = R.slots;
     }
-    if (variant < 0 || variant >= kF64Variants) variant = kF64Variants - 1;
-    S = clamp_split(S, A.tile_hi - A.tile_lo, s, A.part_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *A.split_used = S;
-    const int64_t I = f64_I(variant);
-    const int64_t W = qdiv(s + I - 1, I) * S;
-    for (int64_t w = blockIdx.x; w < W; w += gridDim.x) {
-        const int64_t bx = qdiv(w, S);
-        const int by = (int)(w - bx * S);
-        if (variant == 0)
-            work_f64_stream(A, s, bx, by, S, red);
-        else
-            work_f64_iloop(A, s, bx, by, S);
-        finish_item_f64(A, s, bx, S, I, &last);
+    __syncthreads();
+    const F64Run &R = run;
+    if (blockIdx.x >= R.G) return;
+    const int64_t u1 = R.U * (blockIdx.x + 1) / R.G;
+    for (int64_t u = R.U * blockIdx.x / R.G; u < u1;) {
+        const int64_t b = u / R.units, bu = b * R.units;
+        const int64_t ue = bu + R.units < u1 ? bu + R.units : u1;
+        const int64_t j0 = R.jlo + (u - bu) * R.unit;
+        const int64_t je = R.jlo + (ue - bu) * R.unit;
+        const int64_t j1 = je < R.jhi ? je : R.jhi;
+        const int64_t ib0 = b * R.I;
+        double v;
+        int TJ;
+        switch (R.I) {
+        case 32: v = f64_item<1>(A, s, ib0, j0, j1, sacc); TJ = 1; break;
+        case 16: v = f64_item<2>(A, s, ib0, j0, j1, sacc); TJ = 2; break;
+        case 8: v = f64_item<4>(A, s, ib0, j0, j1, sacc); TJ = 4; break;
+        case 4: v = f64_item<8>(A, s, ib0, j0, j1, sacc); TJ = 8; break;
+        case 2: v = f64_item<16>(A, s, ib0, j0, j1, sacc); TJ = 16; break;
+        default: v = f64_item<32>(A, s, ib0, j0, j1, sacc); TJ = 32; break;
+        }
+        const int lane = tid & 31, warp = tid >> 5;
+        const int64_t ii = ib0 + lane / TJ;
+        const bool holds = warp < 7 && lane % TJ == 0 && ii < s;
+        const int64_t c0 = f64_owner(R, bu);
+        const int n = (int)(f64_owner(R, bu + R.units - 1) - c0) + 1;   // CTAs that meet this i-block
+        if (n == 1) {
+            if (holds) put_final(A, ii, warp, v);
+            __syncthreads();   // sacc is rewritten by the next i-block
+        } else {
+            if (holds) A.part[(ii * R.slots + (blockIdx.x - c0)) * kPartStride + warp] = v;
+            __syncthreads();
+            if (tid == 0) {
+                __threadfence();
+                last = atomicAdd(&A.tickets[b], 1) == n - 1;
+            }
+            __syncthreads();
+            if (last) {
+                __threadfence();
+                f64_finish(A, ib0, (int)(ib0 + R.I < s ? R.I : s - ib0), n, R.slots);
+                if (tid == 0) A.tickets[b] = 0;
+            }
+        }
+        u = ue;
     }
 }
 
@@ -1250,7 +1323,10 @@ void default_tuning(int precision, int64_t n, int64_t s, int num_sms, int ctas_p
     const int64_t resident = (int64_t)num_sms * ctas_per_sm;
     int v;
     if (precision == NB_PREC_FP64) {
-        v = s <= 64 ? 0 : 1;
+        // every CTA of the grid on equal runs of (i-block, j) units
+        *variant = 1;
+        *split = (int)resident;
+        return;
     } else if (mixed_share_fits(n_tiles) && s > 16 && s <= 8192) {
         // the j-records fit the resident shares of a cluster: no split partials in L2
         v = kShareVariant;
@@ -1262,7 +1338,7 @@ void default_tuning(int precision, int64_t n, int64_t s, int num_sms, int ctas_p
         // large N: re-reading all j per i-particle costs more than it hides
         v = s <= 1 ? 0 : s <= 4 ? 1 : s <= 32 ? 2 : s <= 512 ? 3 : 4;
     }
-    const int64_t I = precision == NB_PREC_FP64 ? f64_I(v) : mixed_I(v);
+    const int64_t I = mixed_I(v);
     *variant = v;
     *split = (int)wave_split((s + I - 1) / I, n_tiles, resident);
 }
