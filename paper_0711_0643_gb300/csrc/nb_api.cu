@@ -949,6 +949,7 @@ static PertArgs pert_args(nb_ctx *ctx, int32_t nbin, const int32_t *pairs, doubl
     P.np = ctx->n_pad;
     P.m = ctx->m;
     P.x = ctx->x;
+    P.x2 = ctx->x2;
     P.nbin = nbin;
     P.pairs = pairs;
     P.gamma = gamma;

@@ -92,6 +92,7 @@ struct ForceArgs {
 struct PertArgs {
     int64_t n, np;          // particles, stride of the [3][np] position array
     const double *m, *x;    // masses, positions [3][np]
+    const float2 *x2;       // double-single copy of x
     int32_t nbin;
     const int32_t *pairs;   // [nbin][2] member indices
     double gamma;
