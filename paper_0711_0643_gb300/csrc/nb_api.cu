@@ -325,7 +325,7 @@ nb_status alloc_system(nb_ctx *ctx, int64_t n)
     CK(dalloc(&ctx->a2, 3 * np));
     CK(dalloc(&ctx->k2, 3 * np));
     CK(cudaMemsetAsync(ctx->tickets, 0, (np + 1) * sizeof(int32_t), ctx->stream));
-    ctx->en_ctas = (int)((n + 127) / 128) * 8;   // i-tiles of 128 x up to 8 j-splits
+    ctx->en_ctas = 7 * ctx->num_sms;   // the energy kernel's resident CTAs
     CK(dalloc(&ctx->en_scratch, 2 * (size_t)ctx->en_ctas));
     CK(dalloc(&ctx->out_a, 3 * np));
     CK(dalloc(&ctx->out_k, 3 * np));
@@ -602,7 +602,7 @@ nb_status nb_create(nb_ctx **out, const nb_config *cfg, void *stream)
               dalloc(&ctx->t_end, 1) == cudaSuccess && dalloc(&ctx->split_used, 1) == cudaSuccess &&
               dalloc(&ctx->tune_dev, 1) == cudaSuccess && dalloc(&ctx->status, 1) == cudaSuccess &&
               dalloc(&ctx->counters, 4 + NB_SIZE_BUCKETS) == cudaSuccess && dalloc(&ctx->interactions, 1) == cudaSuccess &&
-              dalloc(&ctx->en_out, 2) == cudaSuccess && dalloc(&ctx->t_eng, 1) == cudaSuccess;
+              dalloc(&ctx->en_out, 3) == cudaSuccess && dalloc(&ctx->t_eng, 1) == cudaSuccess;
     if (!ok) {
         nb_destroy(ctx);
         return NB_ERR_CUDA;
@@ -610,6 +610,7 @@ nb_status nb_create(nb_ctx **out, const nb_config *cfg, void *stream)
     int64_t init_counters[4 + NB_SIZE_BUCKETS] = {0, 0, int64_t(1) << 40};
     int32_t one = 1;
     bool ok2 = cudaMemset(ctx->status, 0, sizeof(int32_t)) == cudaSuccess &&
+               cudaMemset(ctx->en_out, 0, 3 * sizeof(double)) == cudaSuccess &&
                cudaMemcpy(ctx->counters, init_counters, sizeof init_counters, cudaMemcpyHostToDevice) ==
                    cudaSuccess &&
                cudaMemcpy(ctx->split_used, &one, sizeof one, cudaMemcpyHostToDevice) == cudaSuccess &&

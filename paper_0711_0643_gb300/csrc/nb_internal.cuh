@@ -192,9 +192,9 @@ cudaError_t launch_set_active(const int32_t *src, int32_t *dst, int64_t s, int64
 cudaError_t launch_pad_records(const StepArgs &a, cudaStream_t st);
 // caller's forces a[s][3], k[s][3] into the final-sum layout fin[s][8]
 cudaError_t launch_forces_in(const double *a, const double *k, int64_t s, double *fin, cudaStream_t st);
-// energy: writes K, W to out[0], out[1] (fixed-order sums)
-cudaError_t launch_energy(const StepArgs &a, double *scratch, int scratch_ctas, double *out,
-                          cudaStream_t st);
+// energy: writes K, W to out[0], out[1] (fixed-order sums; out[2] is the kernel's arrival
+// counter, zero between launches); scratch: two doubles for each of max_ctas CTAs
+cudaError_t launch_energy(const StepArgs &a, double *scratch, int max_ctas, double *out, cudaStream_t st);
 cudaError_t launch_check_active(const int32_t *idx, int64_t s, int64_t n, int32_t *status,
                                 cudaStream_t st);
 cudaError_t launch_check_due(const StepArgs &a, double t_block, cudaStream_t st);

@@ -10,6 +10,8 @@
 #include <cooperative_groups.h>
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "nb_ds.cuh"
 #include "nb_exact.cuh"
 #include "nb_hermite.cuh"
@@ -641,92 +643,240 @@ __global__ void set_active_kernel(const int32_t *src, int32_t *dst, int64_t s, i
 }
 
 // ------------------------------------------------------------------- energy
-// K = sum m v^2 / 2, W = sum m_i phi_i / 2 with the softened FP64 potential.
-// Each CTA sums its particles in a fixed order into scratch[cta][2]; a single
-// thread then adds the CTA sums in index order.
+// K = sum m v^2 / 2 (FP64) and W = -sum_{i<j} m_i m_j / r_ij, softened, with the pair
+// terms in double-single on the FP32 pipe (an FP64 instruction costs ~64 FP32 lanes'
+// worth here). Every pair once: i-block b (kEnThreads particles, one per thread)
+// takes the j's after its own first particle, in units of kEnUnit j's; the pairs with
+// j <= i of its first kEnThreads j's count as zero. All (i-block, unit) pairs are laid
+// out in one line and cut into equal runs, one per CTA, so every SM has the same work
+// whatever n; FP64 takes over per particle (m_i phi_i), for the CTA's sums and for the
+// total, which the last CTA adds up in CTA order (fixed order: the same bits on
+// every run).
+//
+// What bounds it: ~87 packed f32x2 operations per pair of j's, i.e. the FP32 pipe and
+// the operand reads from the register file (two 32-bit operands per lane and clock).
+// N = 32768: 4485 us with every pair evaluated twice, scalar (135 issue slots a pair,
+// issue-bound) and a one-thread final sum of 157 us; now 1430 us (N = 1000: 65 -> 37).
 constexpr int kEnThreads = 128;
-constexpr int kEnSplitMax = 8;   // j-splits per i-tile (the scratch holds that many partials per tile)
+constexpr int kEnUnit = 32;
 
-// K and W of the current state. Grid (i-tiles of 128, j-splits): each thread
-// sums m_j / r_ij over its split's j != i in double-single on the FP32 pipe (an
-// FP64 instruction costs ~64 FP32 lanes' worth here); FP64 takes over per
-// particle (W_i = -m_i phi_i / 2, K_i = m_i v_i^2 / 2) and for the CTA and final
-// sums, all in a fixed order.
-__global__ void __launch_bounds__(kEnThreads) energy_kernel(StepArgs A, double *scratch, int S)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
 {
-    __shared__ float4 sj[kEnThreads][2];
-    __shared__ double sk[kEnThreads / 32], sw[kEnThreads / 32];
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+    return *reinterpret_cast<float2 *>(&r);
+}
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+
+// s + e = a + b exactly (Knuth's two-sum)
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2 &s, float2 &e)
+{
+    s = __fadd2_rn(a, b);
+    const float2 bb = sub2(s, a);
+    e = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+
+// h + l = (ah + al) - (bh + bl), normalised
+__device__ __forceinline__ void diff2(float2 ah, float2 al, float2 bh, float2 bl, float2 &h, float2 &l)
+{
+    const float2 s = sub2(ah, bh);
+    const float2 bb = sub2(s, ah);
+    float2 e = sub2(sub2(ah, sub2(s, bb)), __fadd2_rn(bh, bb));
+    e = __fadd2_rn(e, sub2(al, bl));
+    h = __fadd2_rn(s, e);
+    l = sub2(e, sub2(h, s));
+}
+
+struct EnI {
+    float2 xh, xl, yh, yl, zh, zl;   // a particle's double-single position, in both lanes
+};
+
+// (h, l) -= m_j / r_ij for the two j's of a shared-memory record (q0: x_hi, x_hi',
+// y_hi, y_hi'; q1: z_hi, z_hi', m_hi, m_hi'; q2, q3 the low parts): r from the
+// double-single positions, r^2 + eps^2 with exact squares and two-sums (within 2^-45),
+// y = (r^2 + eps^2)^(-1/2) from the hardware estimate and a third-order step on the
+// residual 1 - r^2 y^2, which is formed to 2^-46. MASK: zero for lanes with keep unset.
+template <bool MASK>
+__device__ __forceinline__ void en_pair2(const float4 &q0, const float4 &q1, const float4 &q2, const float4 &q3,
+                                         const EnI &I, float2 e2h, float2 e2l, bool keep_a, bool keep_b, float2 &h,
+                                         float2 &l)
+{
+    float2 dx, lx, dy, ly, dz, lz;
+    diff2(make_float2(q0.x, q0.y), make_float2(q2.x, q2.y), I.xh, I.xl, dx, lx);
+    diff2(make_float2(q0.z, q0.w), make_float2(q2.z, q2.w), I.yh, I.yl, dy, ly);
+    diff2(make_float2(q1.x, q1.y), make_float2(q3.x, q3.y), I.zh, I.zl, dz, lz);
+    const float2 px = __fmul2_rn(dx, dx), py = __fmul2_rn(dy, dy), pz = __fmul2_rn(dz, dz);
+    float2 low = __fadd2_rn(__fadd2_rn(__ffma2_rn(dx, dx, neg2(px)), __ffma2_rn(dy, dy, neg2(py))),
+                            __ffma2_rn(dz, dz, neg2(pz)));
+    const float2 cross = __ffma2_rn(dx, lx, __ffma2_rn(dy, ly, __fmul2_rn(dz, lz)));
+    low = __ffma2_rn(dup2(2.f), cross, low);
+    float2 s, e;
+    two_sum2(px, py, s, e);
+    low = __fadd2_rn(low, e);
+    two_sum2(s, pz, s, e);
+    low = __fadd2_rn(low, e);
+    two_sum2(s, e2h, s, e);
+    low = __fadd2_rn(__fadd2_rn(low, e2l), e);
+    // s + low = r^2 + eps^2
+    const float2 y = make_float2(rsqrtf(s.x), rsqrtf(s.y));
+    const float2 ny = neg2(y);
+    const float2 nt = __fmul2_rn(s, ny);
+    const float2 te = __ffma2_rn(low, y, __ffma2_rn(s, y, nt));
+    const float2 res = __ffma2_rn(te, ny, __ffma2_rn(nt, y, dup2(1.f)));
+    const float2 ql = __fmul2_rn(y, __fmul2_rn(res, __ffma2_rn(res, dup2(0.375f), dup2(0.5f))));
+    const float2 mh = make_float2(q1.z, q1.w), ml = make_float2(q3.z, q3.w);
+    float2 th = __fmul2_rn(mh, ny);
+    float2 tl = __ffma2_rn(ml, y, __ffma2_rn(mh, ql, __ffma2_rn(mh, y, th)));   // -(low part)
+    if (MASK) {
+        th.x = keep_a ? th.x : 0.f;
+        tl.x = keep_a ? tl.x : 0.f;
+        th.y = keep_b ? th.y : 0.f;
+        tl.y = keep_b ? tl.y : 0.f;
+    }
+    two_sum2(h, th, h, e);
+    l = __fadd2_rn(l, sub2(e, tl));
+}
+
+// Units of the i-blocks before b (block q has nu - 4 q units)
+__device__ __forceinline__ int64_t en_before(int64_t b, int64_t nu)
+{
+    return b * nu - (kEnThreads / kEnUnit) * (b * (b - 1) / 2);
+}
+
+__global__ void __launch_bounds__(kEnThreads, 7) energy_kernel(StepArgs A, double *scratch, double *out)
+{
+    __shared__ float4 sj[4][kEnThreads / 2];
+    __shared__ double red[2][kEnThreads / 32];
+    __shared__ int last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n = A.n, np = A.n_pad;
-    const int64_t i = (int64_t)blockIdx.x * kEnThreads + threadIdx.x;
-    const int by = blockIdx.y;
-    const bool live = i < n;
-    const int64_t ii = live ? i : 0;
-    const float2 xi = rn_ds_pack(A.x[ii]), yi = rn_ds_pack(A.x[np + ii]), zi = rn_ds_pack(A.x[2 * np + ii]);
-    const float2 e2 = rn_ds_pack(A.eps2);
-    float ph = 0.f, pl = 0.f;
-    const int64_t ntile = (n + kEnThreads - 1) / kEnThreads;
-    const int64_t per = (ntile + S - 1) / S;
-    const int64_t t0 = (int64_t)by * per;
-    const int64_t t1 = t0 + per < ntile ? t0 + per : ntile;
-    for (int64_t t = t0; t < t1; ++t) {
-        const int64_t j = t * kEnThreads + threadIdx.x;
-        __syncthreads();
-        if (j < n) {
-            const float2 x = rn_ds_pack(A.x[j]), y = rn_ds_pack(A.x[np + j]), z = rn_ds_pack(A.x[2 * np + j]);
-            const float2 m = rn_ds_pack(A.m[j]);
-            sj[threadIdx.x][0] = make_float4(x.x, x.y, y.x, y.y);
-            sj[threadIdx.x][1] = make_float4(z.x, z.y, m.x, m.y);
-        }
-        __syncthreads();
-        const int jn = (int)(n - t * kEnThreads < kEnThreads ? n - t * kEnThreads : kEnThreads);
-        const int self = (int)(i - t * kEnThreads);   // tile slot of i, if it is in this tile
-        for (int q = 0; q < jn; ++q) {
-            float th, tl;
-            en_pair(sj[q][0], sj[q][1], xi, yi, zi, e2, th, tl);
-            if (q != self) en_acc(ph, pl, th, tl);
+    const int64_t nblk = (n + kEnThreads - 1) / kEnThreads, nu = (n + kEnUnit - 1) / kEnUnit;
+    const int64_t U = en_before(nblk, nu);
+    const int64_t u1 = U * (blockIdx.x + 1) / gridDim.x;
+    int64_t u = U * blockIdx.x / gridDim.x;
+    // the i-block of unit u
+    int64_t b = 0;
+    {
+        int64_t hi = nblk;   // en_before(b) <= u < en_before(hi)
+        while (hi - b > 1) {
+            const int64_t mid = (b + hi) / 2;
+            if (en_before(mid, nu) <= u)
+                b = mid;
+            else
+                hi = mid;
         }
     }
+    const float2 e2 = rn_ds_pack(A.eps2);
+    const float2 e2h = dup2(e2.x), e2l = dup2(e2.y);
     double ek = 0.0, ew = 0.0;
-    if (live) {
-        const double mi = A.m[i];
-        ew = -0.5 * mi * ((double)ph + (double)pl);
-        if (by == 0) {
-            const double vx = A.v[i], vy = A.v[np + i], vz = A.v[2 * np + i];
-            ek = 0.5 * mi * (vx * vx + vy * vy + vz * vz);
+    while (u < u1) {
+        const int64_t first = en_before(b, nu), end = en_before(b + 1, nu);
+        const int64_t ue = end < u1 ? end : u1;
+        const int64_t i0 = b * kEnThreads, i = i0 + tid;
+        const bool live = i < n;
+        const int64_t ii = live ? i : 0;
+        const float2 x = A.x2[ii], y = A.x2[np + ii], z = A.x2[2 * np + ii];
+        const EnI I{dup2(x.x), dup2(x.y), dup2(y.x), dup2(y.y), dup2(z.x), dup2(z.y)};
+        float2 h = dup2(0.f), l = dup2(0.f);
+        const int64_t j0 = i0 + (u - first) * kEnUnit, je = i0 + (ue - first) * kEnUnit;
+        const int64_t j1 = je < n ? je : n;
+        for (int64_t jt = j0; jt < j1; jt += kEnThreads) {
+            __syncthreads();
+            {
+                const int64_t j = jt + tid;
+                const bool real = j < j1;   // massless far-away records past the end add exact zeros
+                const float far = (float)kPadPos;
+                const float2 xj = real ? A.x2[j] : make_float2(far, 0.f), yj = real ? A.x2[np + j] : make_float2(far, 0.f),
+                             zj = real ? A.x2[2 * np + j] : make_float2(far, 0.f);
+                const float2 mj = real ? rn_ds_pack(A.m[j]) : make_float2(0.f, 0.f);
+                float *q = reinterpret_cast<float *>(&sj[0][tid >> 1]) + (tid & 1);
+                constexpr int kRow = 4 * (kEnThreads / 2);
+                q[0] = xj.x;
+                q[2] = yj.x;
+                q[kRow] = zj.x;
+                q[kRow + 2] = mj.x;
+                q[2 * kRow] = xj.y;
+                q[2 * kRow + 2] = yj.y;
+                q[3 * kRow] = zj.y;
+                q[3 * kRow + 2] = mj.y;
+            }
+            __syncthreads();
+            const int64_t left = j1 - jt;
+            const int np2 = (int)((left < kEnThreads ? left : kEnThreads) + 1) / 2;
+            if (jt < i0 + kEnThreads) {
+                for (int q = 0; q < np2; ++q)
+                    en_pair2<true>(sj[0][q], sj[1][q], sj[2][q], sj[3][q], I, e2h, e2l, jt + 2 * q > i,
+                                   jt + 2 * q + 1 > i, h, l);
+            } else {
+                for (int q = 0; q < np2; ++q)
+                    en_pair2<false>(sj[0][q], sj[1][q], sj[2][q], sj[3][q], I, e2h, e2l, true, true, h, l);
+            }
         }
+        if (live) {
+            const double mi = A.m[i];
+            ew += mi * (((double)h.x + (double)h.y) + ((double)l.x + (double)l.y));
+            if (u == first) {   // the CTA that begins an i-block adds its kinetic energy
+                const double vx = A.v[i], vy = A.v[np + i], vz = A.v[2 * np + i];
+                ek += 0.5 * mi * (vx * vx + vy * vy + vz * vz);
+            }
+        }
+        u = ue;
+        ++b;
     }
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) {
         ek += __shfl_down_sync(0xffffffffu, ek, off);
         ew += __shfl_down_sync(0xffffffffu, ew, off);
     }
-    if ((threadIdx.x & 31) == 0) {
-        sk[threadIdx.x >> 5] = ek;
-        sw[threadIdx.x >> 5] = ew;
+    if (lane == 0) {
+        red[0][warp] = ek;
+        red[1][warp] = ew;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         double K = 0.0, W = 0.0;
         for (int w = 0; w < kEnThreads / 32; ++w) {
-            K += sk[w];
-            W += sw[w];
+            K += red[0][w];
+            W += red[1][w];
         }
-        const int64_t slot = (int64_t)blockIdx.x * S + by;
-        scratch[2 * slot] = K;
-        scratch[2 * slot + 1] = W;
+        scratch[2 * blockIdx.x] = K;
+        scratch[2 * blockIdx.x + 1] = W;
+        __threadfence();
+        // out[2] holds the arrival counter, zero between launches
+        last = atomicAdd(reinterpret_cast<int *>(out + 2), 1) == (int)gridDim.x - 1;
     }
-}
-
-__global__ void energy_final_kernel(const double *scratch, int64_t nslots, double *out)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // the CTA sums in a fixed order: thread t adds slots t, t + kEnThreads, ..., then a tree
+    ek = ew = 0.0;
+    for (int q = tid; q < (int)gridDim.x; q += kEnThreads) {
+        const double2 v = __ldcg(reinterpret_cast<const double2 *>(scratch) + q);
+        ek += v.x;
+        ew += v.y;
+    }
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+        ek += __shfl_down_sync(0xffffffffu, ek, off);
+        ew += __shfl_down_sync(0xffffffffu, ew, off);
+    }
+    if (lane == 0) {
+        red[0][warp] = ek;
+        red[1][warp] = ew;
+    }
+    __syncthreads();
+    if (tid == 0) {
         double K = 0.0, W = 0.0;
-        for (int64_t b = 0; b < nslots; ++b) {
-            K += scratch[2 * b];
-            W += scratch[2 * b + 1];
+        for (int w = 0; w < kEnThreads / 32; ++w) {
+            K += red[0][w];
+            W += red[1][w];
         }
         out[0] = K;
         out[1] = W;
+        *reinterpret_cast<int *>(out + 2) = 0;
     }
 }
 
@@ -939,18 +1089,12 @@ cudaError_t launch_set_active(const int32_t *src, int32_t *dst, int64_t s, int64
     return cudaGetLastError();
 }
 
-cudaError_t launch_energy(const StepArgs &a, double *scratch, int scratch_ctas, double *out, cudaStream_t st)
+cudaError_t launch_energy(const StepArgs &a, double *scratch, int max_ctas, double *out, cudaStream_t st)
 {
-    const int64_t nbx = (a.n + kEnThreads - 1) / kEnThreads;
-    // j-splits so that the grid covers the GPU several times over; the scratch
-    // holds kEnSplitMax partials per i-tile
-    int64_t S = (1216 + nbx - 1) / nbx;
-    if (S > kEnSplitMax) S = kEnSplitMax;
-    if (S > nbx) S = nbx;
-    if (S < 1) S = 1;
-    if (nbx * S > scratch_ctas) return cudaErrorInvalidValue;
-    energy_kernel<<<dim3((unsigned)nbx, (unsigned)S), kEnThreads, 0, st>>>(a, scratch, (int)S);
-    energy_final_kernel<<<1, 32, 0, st>>>(scratch, nbx * S, out);
+    // one run per CTA, at most max_ctas (the scratch holds two sums for each) and one per unit
+    const int64_t nblk = (a.n + kEnThreads - 1) / kEnThreads, nu = (a.n + kEnUnit - 1) / kEnUnit;
+    const int64_t U = nblk * nu - (kEnThreads / kEnUnit) * (nblk * (nblk - 1) / 2);
+    energy_kernel<<<(unsigned)std::min<int64_t>(U, max_ctas), kEnThreads, 0, st>>>(a, scratch, out);
     return cudaGetLastError();
 }
 
