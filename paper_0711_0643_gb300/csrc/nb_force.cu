@@ -3,18 +3,13 @@
 // derivative, and the softened potential.
 //
 // The paper splits the j-sum over processors and adds the partial forces with
-// MPI_Allreduce (Sect. 3). Here the split is on one chip:
-//   * a work item = (i-block, j-split); every CTA of a persistent grid loops
-//     over work items derived on the device from the active count s, so the
-//     launch needs no host round trip and can live inside a CUDA graph;
-//   * j-records stream through shared memory in tiles of kJT records, copied
-//     by the TMA bulk engine (cp.async.bulk + mbarrier, kStages in flight);
-//   * each thread holds R i-particles in registers and sweeps the tile with
-//     TJ threads sharing each i (TJ > 1 splits j inside the CTA when s is small);
-//   * partials are reduced in a fixed order (lane shuffles, then the split
-//     index): the last CTA to finish an i-block (an arrival ticket, no waiting)
-//     sums that block's split partials in ascending split order, so results
-//     are bitwise reproducible run to run.
+// MPI_Allreduce (Sect. 3). Here the split is on one chip: every CTA of a persistent
+// grid derives its share of the work from the active count s on the device, so the
+// launch needs no host round trip and can live inside a CUDA graph; j-records stream
+// through shared memory, copied by the TMA bulk engine (cp.async.bulk + mbarrier);
+// partials are reduced in a fixed order (lane shuffles, then the CTAs' partials): the
+// last CTA to finish an i-block (an arrival ticket, no waiting) adds them, so results
+// are bitwise reproducible run to run.
 //
 // Mixed precision: positions arrive as double-single (hi, lo) pairs so that
 // r = x_j - x_i keeps ~46 bits even for close pairs (velocities are FP32: the
@@ -61,6 +56,11 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
                  : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // 1-D bulk copy global -> shared, completion counted on the mbarrier (TMA).
 // Both addresses 16-byte aligned, size a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
@@ -99,10 +99,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int64_
 
 // ------------------------------------------------------------ shared memory
 
-constexpr int kMaxRC = 2 * 7;   // R * components, largest R over variants
-
 constexpr int kPT = kJT / 2;    // pair records per tile
 constexpr int kRing = 6;        // tiles in flight in the TMA streaming variant
+
+// Column kernel (see there): a unit is up to kUnitRec pair records in kUnitBytes of
+// shared memory, kSlots units in flight.
+constexpr int kUnitRec = 256;
+constexpr int kUnitBytes = kUnitRec * (int)sizeof(JPair);
+constexpr int kSlots = 4;
+constexpr int kShortTiles = 32; // shares of up to this many tiles may go by whole items (see short_items)
 
 // Resident-share variant: clusters of kShareC CTAs, CTA r holding up to
 // kShareRec pair records of the j range in shared memory, the active list dealt
@@ -111,22 +116,42 @@ constexpr int kShareC = 8;
 constexpr int kShareRec = 1024;
 constexpr int kShareSlots = 256;
 
+// How the column kernel cuts a launch (worked out by one thread per CTA).
+struct ColPlan {
+    int64_t tper;       // tiles per share of the table's split
+    int64_t upi;        // units per i-block
+    int64_t nib, U, G;  // i-blocks, units in all, CTAs sharing them
+    int64_t u0, u1, b0; // this CTA's run of units, the i-block it begins in
+    int ups;            // units per share
+    int lgst, lgcw;     // log2 of the column stride (records) and of the columns per unit
+    int lgtj;           // log2 of the threads per i-particle
+    int slots;          // partial slots per particle
+    int whole;          // no i-block is shared between CTAs
+    int part_n, part_slot;   // the current i-block: CTAs that meet it, this one's place
+};
+
 // The staging buffers come last, so that the resident-share variant's larger
-// buffer can take their place and run past the end of the struct: the kernel
-// instantiation without that variant is launched with sizeof(Smem) bytes, the
-// one with it with kSmemShare bytes.
+// buffer can take their place and run past the end of the struct.
 struct __align__(128) Smem {
-    float2 red[kThreads / 32][kMaxRC];
+    float2 red[kThreads / 32][14];
     uint64_t bar[kRing];
     uint64_t inject_bar;
     int64_t s;                 // active count of this launch
+    int64_t items, tper;       // streamed variants: work items, tiles per item,
+    int split, lgi;            //   items per i-block, log2 of the particles of an i-block
     Tuning tune;               // the device tuning table, read once per CTA
     int32_t idx_pre[kThreads]; // the first kThreads entries of the active list, read with s
+    ColPlan plan;              // kept here and not in registers: the pair loop needs those
+    uint64_t empty[kSlots];    // column kernel: every warp has read the slot's unit
+    int2 info[kSlots];         // the unit's rows and columns
     int abort;
     int last;
     alignas(128) union {
-        JPair tile[kStages][kPT];   // tile variants
-        JPair ring[kRing][kPT];     // TMA streaming variant
+        JPair ring[kRing][kPT];                      // TMA streaming variant
+        struct {
+            unsigned char unit[kSlots][kUnitBytes];  // column kernel
+            float2 sums[7][kThreads];                // its threads' sums of an i-block
+        };
     };
 };
 
@@ -135,9 +160,10 @@ struct ShareBuf {
     float2 slot[kShareSlots][7];     // (hi, lo) partials of the chunk's particles
 };
 
-constexpr size_t kSmemShare = (offsetof(Smem, tile) + sizeof(ShareBuf) + 127) / 128 * 128;
+constexpr size_t kSmemShare =
+    (sizeof(Smem) > offsetof(Smem, ring) + sizeof(ShareBuf) ? sizeof(Smem) : offsetof(Smem, ring) + sizeof(ShareBuf));
 
-__device__ __forceinline__ ShareBuf *shb(Smem *sm) { return reinterpret_cast<ShareBuf *>(&sm->tile[0][0]); }
+__device__ __forceinline__ ShareBuf *shb(Smem *sm) { return reinterpret_cast<ShareBuf *>(&sm->ring[0][0]); }
 
 __device__ __forceinline__ int bucket_of(int64_t s)
 {
@@ -156,14 +182,17 @@ __device__ __forceinline__ int64_t qdiv(int64_t a, int64_t b)
     return a / b;
 }
 
+__device__ __forceinline__ int64_t qmod(int64_t a, int64_t b) { return a - qdiv(a, b) * b; }
+
 // The table's split is the one for its bucket's largest size s_ref = min(2^b, n);
 // a smaller block of the bucket keeps the same number of work items (i-blocks x
 // splits), so a wave-aligned choice stays wave-aligned.
 __device__ __forceinline__ int table_split(int S_ref, int b, int64_t s, int64_t n, int64_t I)
 {
     const int64_t s_ref = (int64_t(1) << b) < n ? (int64_t(1) << b) : n;
-    const int64_t nib_ref = qdiv(s_ref + I - 1, I), nib = qdiv(s + I - 1, I);
-    const int64_t S = qdiv((int64_t)S_ref * nib_ref, nib);
+    const int lg = 31 - __clz((int)I);   // I is a power of two
+    const int64_t nib_ref = (s_ref + I - 1) >> lg, nib = (s + I - 1) >> lg;
+    const int64_t S = nib_ref == nib ? S_ref : qdiv((int64_t)S_ref * nib_ref, nib);
     return S < 1 ? 1 : (S > (1 << 30) ? (1 << 30) : (int)S);
 }
 
@@ -178,9 +207,10 @@ __device__ __forceinline__ int clamp_split(int S, int64_t n_tiles, int64_t s, in
 {
     if (S < 1) S = 1;
     if (S > n_tiles) S = (int)n_tiles;
-    int64_t lim = qdiv(cap, s * kPartStride);
-    if (lim < 1) lim = 1;
-    if (S > lim) S = (int)lim;
+    if ((int64_t)S * s * kPartStride > cap) {
+        const int64_t lim = qdiv(cap, s * kPartStride);
+        S = lim < 1 ? 1 : (int)lim;
+    }
     return S;
 }
 
@@ -188,14 +218,6 @@ __device__ __forceinline__ int clamp_split(int S, int64_t n_tiles, int64_t s, in
 __device__ __forceinline__ float2 *part2(const ForceArgs &A, int64_t ii, int by, int S)
 {
     return reinterpret_cast<float2 *>(A.part) + (ii * S + by) * kPartStride;
-}
-
-__device__ __forceinline__ void write_part(const ForceArgs &A, int64_t ii, int by, int S, const Acc7 &hi,
-                                           const Acc7 &lo)
-{
-    float2 *dst = part2(A, ii, by, S);
-#pragma unroll
-    for (int c = 0; c < 7; ++c) dst[c] = make_float2(acc_get(hi, c), acc_get(lo, c));
 }
 
 // Final sum of component c (ax ay az kx ky kz phi) of active particle ii: into
@@ -222,118 +244,151 @@ __device__ __forceinline__ void copy_list(const ForceArgs &A, int64_t s)
     if (blockIdx.x == 0 && threadIdx.x == 0) *A.s_copy = s;
 }
 
-// Called by every thread after a work item has written its partials. The CTA
-// that completes the i-block (ticket S - 1) adds the block's S partials in split
-// order with two-sums and writes the FP64 results; it then re-arms the ticket.
-__device__ void finish_item(const ForceArgs &A, int64_t s, int64_t bx, int S, int64_t I, Smem *sm)
+// Adds the n partials of each of the active particles [ib0, ib1) (slots 0 .. n - 1 of S)
+// by this CTA, in a fixed order, and writes the results.
+__device__ void sum_parts(const ForceArgs &A, int64_t ib0, int64_t ib1, int S, int n)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int np = (int)(ib1 - ib0);
+    if (np == 1) {
+        // a warp per component; lane l adds partials l, l + 32, ... (kUnroll loads per
+        // round), then a butterfly of two-sums over the lanes
+        constexpr int kUnroll = 4;
+        if (warp < 7) {
+            const float2 *src = part2(A, ib0, 0, S) + warp;
+            float h = 0.f, l = 0.f;
+            for (int q0 = lane; q0 < n; q0 += 32 * kUnroll) {
+                float2 v[kUnroll];
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u)
+                    v[u] = q0 + 32 * u < n ? __ldcg(src + (q0 + 32 * u) * kPartStride) : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u)
+                    if (q0 + 32 * u < n) ds_add(h, l, v[u].x, v[u].y);
+            }
+            ds_group_reduce<32>(h, l);
+            if (lane == 0) put_final(A, ib0, warp, (double)h + (double)l);
+        }
+        return;
+    }
+    // D threads per (particle, component pair), neighbours in a warp, thread d adding
+    // partials d, d + D, ... with kLoads 16-byte loads issued together (an L2 round trip
+    // each: the sum is bound by how many are in flight), then a tree over the D threads.
+    constexpr int kLoads = 16;
+    const int D = np <= 8 ? 8 : (np <= 16 ? 4 : (np <= 32 ? 2 : 1));
+    const int qc = threadIdx.x & 3, d = (threadIdx.x >> 2) & (D - 1);
+    const int per = kThreads / (4 * D);   // particles at a time
+    for (int p0 = 0; p0 < np; p0 += per) {
+        const int pi = p0 + threadIdx.x / (4 * D);
+        const int64_t ii = ib0 + (pi < np ? pi : np - 1);
+        const float4 *src = reinterpret_cast<const float4 *>(part2(A, ii, 0, S)) + qc;
+        float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+        for (int q0 = d; q0 < n; q0 += D * kLoads) {
+            float4 v[kLoads];
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u) {
+                const int q = q0 + D * u;
+                v[u] = q < n ? __ldcg(src + q * (kPartStride / 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u)
+                if (q0 + D * u < n) {
+                    ds_add(h0, l0, v[u].x, v[u].y);
+                    if (qc < 3) ds_add(h1, l1, v[u].z, v[u].w);   // component 7 is padding
+                }
+        }
+        for (int off = 4; off < 4 * D; off <<= 1) {
+            const float a0 = __shfl_xor_sync(0xffffffffu, h0, off), b0 = __shfl_xor_sync(0xffffffffu, l0, off);
+            const float a1 = __shfl_xor_sync(0xffffffffu, h1, off), b1 = __shfl_xor_sync(0xffffffffu, l1, off);
+            ds_add(h0, l0, a0, b0);
+            ds_add(h1, l1, a1, b1);
+        }
+        if (d == 0 && pi < np) {
+            put_final(A, ii, 2 * qc, (double)h0 + (double)l0);
+            if (qc < 3) put_final(A, ii, 2 * qc + 1, (double)h1 + (double)l1);
+        }
+    }
+}
+
+// Called by every thread after this CTA has written its partials of i-block bx (active
+// particles [ib0, ib1)). The CTA that completes the block's n partials (ticket n - 1)
+// adds them with two-sums and writes the FP64 results; it then re-arms the ticket.
+__device__ void finish_block(const ForceArgs &A, int64_t bx, int64_t ib0, int64_t ib1, int S, int n, Smem *sm)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         const int t = atomicAdd(&A.tickets[bx], 1);
-        sm->last = (t == S - 1);
+        sm->last = (t == n - 1);
     }
     __syncthreads();
     if (sm->last) {
         __threadfence();
-        const int64_t ib0 = bx * I;
-        const int64_t ib1 = ib0 + I < s ? ib0 + I : s;
-        const int cnt = (int)(ib1 - ib0) * 7;
-        if (S <= 4) {
-            // few splits: one thread per (particle, component)
-            for (int q = threadIdx.x; q < cnt; q += kThreads) {
-                const int64_t ii = ib0 + q / 7;
-                const int c = q % 7;
-                const float2 *src = reinterpret_cast<const float2 *>(A.part) + ii * S * kPartStride + c;
-                float h = 0.f, l = 0.f;
-                for (int sp = 0; sp < S; ++sp) {
-                    const float2 v = __ldcg(src + sp * kPartStride);
-                    ds_add(h, l, v.x, v.y);
-                }
-                put_final(A, ii, c, (double)h + (double)l);
-            }
-        } else {
-            // many splits. The order of every addition is the split order per lane, then a
-            // fixed tree over lanes, so the batching of the loads does not change the result.
-            constexpr int kFinUnroll = 4;
-            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-            const float2 *base = reinterpret_cast<const float2 *>(A.part);
-            if (cnt <= kThreads / 32) {
-                // one particle: a warp per component; lane l adds splits l, l + 32, ...
-                // (kFinUnroll loads per round), then a butterfly of two-sums over the lanes
-                if (warp < cnt) {
-                    const float2 *src = base + (ib0 + warp / 7) * S * kPartStride + warp % 7;
-                    float h = 0.f, l = 0.f;
-                    for (int sp0 = lane; sp0 < S; sp0 += 32 * kFinUnroll) {
-                        float2 v[kFinUnroll];
-#pragma unroll
-                        for (int u = 0; u < kFinUnroll; ++u)
-                            v[u] = sp0 + 32 * u < S ? __ldcg(src + (sp0 + 32 * u) * kPartStride) : make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int u = 0; u < kFinUnroll; ++u)
-                            if (sp0 + 32 * u < S) ds_add(h, l, v[u].x, v[u].y);
-                    }
-                    ds_group_reduce<32>(h, l);
-                    if (lane == 0) put_final(A, ib0 + warp / 7, warp % 7, (double)h + (double)l);
-                }
-            } else {
-                // a warp per particle: the particle's S partials are S x 64 contiguous
-                // bytes, read with 16-byte loads (kFinLoads issued together). Lane l takes
-                // components 2 (l % 4) and 2 (l % 4) + 1 of splits l / 4, l / 4 + 8, ... and
-                // adds them in ascending split order; a fixed tree over the eight lanes of
-                // each component pair (lane distance 4, 8, 16) finishes the sum.
-                constexpr int kFinLoads = 16;
-                const int qc = lane & 3, sub = lane >> 2;
-                const int np = (int)(ib1 - ib0);
-                for (int pi = warp; pi < np; pi += kThreads / 32) {
-                    const int64_t ii = ib0 + pi;
-                    const float4 *src = reinterpret_cast<const float4 *>(A.part) + ii * S * (kPartStride / 2) + qc;
-                    float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
-                    for (int sp0 = sub; sp0 < S; sp0 += 8 * kFinLoads) {
-                        float4 v[kFinLoads];
-#pragma unroll
-                        for (int u = 0; u < kFinLoads; ++u) {
-                            const int sp = sp0 + 8 * u;
-                            v[u] = sp < S ? __ldcg(src + (int64_t)sp * (kPartStride / 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-#pragma unroll
-                        for (int u = 0; u < kFinLoads; ++u)
-                            if (sp0 + 8 * u < S) {
-                                ds_add(h0, l0, v[u].x, v[u].y);
-                                if (qc < 3) ds_add(h1, l1, v[u].z, v[u].w);   // component 7 is padding
-                            }
-                    }
-#pragma unroll
-                    for (int off = 4; off <= 16; off <<= 1) {
-                        const float a0 = __shfl_xor_sync(0xffffffffu, h0, off), b0 = __shfl_xor_sync(0xffffffffu, l0, off);
-                        const float a1 = __shfl_xor_sync(0xffffffffu, h1, off), b1 = __shfl_xor_sync(0xffffffffu, l1, off);
-                        ds_add(h0, l0, a0, b0);
-                        ds_add(h1, l1, a1, b1);
-                    }
-                    if (sub == 0) {
-                        put_final(A, ii, 2 * qc, (double)h0 + (double)l0);
-                        if (qc < 3) put_final(A, ii, 2 * qc + 1, (double)h1 + (double)l1);
-                    }
-                }
-            }
-        }
+        sum_parts(A, ib0, ib1, S, n);
         if (threadIdx.x == 0) A.tickets[bx] = 0;
     }
     __syncthreads();
 }
 
 // ------------------------------------------------------- streamed variant
-// TI = 1: all threads share the same R i-particles; each thread walks its own
-// pair records straight from global memory (coalesced float4 loads), so no
-// shared staging is needed. For small active blocks.
-template <int R>
-__device__ void work_stream(const ForceArgs &A, int64_t s, int64_t bx, int by, int S, Smem *sm)
+// All threads share the same R i-particles; each thread walks its own pair records
+// straight from global memory, so no shared staging is needed. For the smallest active
+// blocks: a call is then a chain of latencies, and this chain is the shortest.
+
+// Item w of the launch: i-block bx and tiles [t0, t1) (the launch's split and tiles per
+// item are kept in shared memory: the pair loops need the registers).
+__device__ __forceinline__ void stream_item(const ForceArgs &A, int64_t w, const Smem *sm, int64_t &bx, int64_t &t0,
+                                            int64_t &t1)
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t tper = qdiv(A.tile_hi - A.tile_lo + S - 1, S);
-    const int64_t t0 = A.tile_lo + (int64_t)by * tper;
-    const int64_t t1 = t0 + tper < A.tile_hi ? t0 + tper : A.tile_hi;
-    const int64_t p0 = t0 * kPT, p1 = t1 * kPT;
+    bx = qdiv(w, sm->split);
+    const int64_t by = w - bx * sm->split;
+    t0 = A.tile_lo + by * sm->tper;
+    t1 = t0 + sm->tper < A.tile_hi ? t0 + sm->tper : A.tile_hi;
+}
+
+// The CTA's sums of particle bx, r-th of the CTA's: into the CTA's partial slot or,
+// where the CTA holds all of j (S == 1), the results.
+__device__ __forceinline__ void cta_sum_red(const Acc7 &hi, const Acc7 &lo, float2 *red)
+{
+    float h, l;
+    const int lane = threadIdx.x & 31;
+    const int c = ds_scatter_reduce<32>(hi, lo, h, l);   // a lane holds component c
+    if ((lane & 3) == 0 && c < 7) red[c] = make_float2(h, l);
+}
+template <int R>
+__device__ __forceinline__ void cta_sum_out(const ForceArgs &A, int64_t w, Smem *sm)
+{
+    // warps in ascending order
+    const int tid = threadIdx.x, S = sm->split;
+    const int64_t s = sm->s, bx = qdiv(w, S), i0 = bx * R;
+    const int by = (int)(w - bx * S);
+    if (tid < 7 * R) {
+        float h = sm->red[0][tid].x, l = sm->red[0][tid].y;
+#pragma unroll
+        for (int wv = 1; wv < kThreads / 32; ++wv) ds_add(h, l, sm->red[wv][tid].x, sm->red[wv][tid].y);
+        const int64_t ii = i0 + tid / 7;
+        const int c = tid % 7;
+        if (ii < s) {
+            if (S == 1)
+                put_final(A, ii, c, (double)h + (double)l);
+            else
+                part2(A, ii, by, S)[c] = make_float2(h, l);
+        }
+    }
+}
+
+template <int R>
+__device__ void work_stream(const ForceArgs &A, int64_t w, Smem *sm)
+{
+    const int tid = threadIdx.x, warp = tid >> 5;
+    int64_t bx;
+    int p0, p1;   // records: fewer than 2^30
+    {
+        int64_t t0, t1;
+        stream_item(A, w, sm, bx, t0, t1);
+        p0 = (int)(t0 * kPT);
+        p1 = (int)(t1 * kPT);
+    }
     // this thread's first pair record moves into L1 while the i-particle loads
     // are in flight (a prefetch holds no registers)
     if (p0 + tid < p1) {
@@ -345,8 +400,8 @@ __device__ void work_stream(const ForceArgs &A, int64_t s, int64_t bx, int by, i
     int32_t gi[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        int64_t ii = bx * R + r;
-        gi[r] = idx_at(A, sm, ii < s ? ii : s - 1);
+        const int64_t ii = bx * R + r;
+        gi[r] = idx_at(A, sm, ii < sm->s ? ii : sm->s - 1);
         ip[r] = ipk_of(jrec_load(A.j.p, gi[r]));
     }
     const float2 e2 = make_float2(A.eps2f, A.eps2f);
@@ -354,11 +409,13 @@ __device__ void work_stream(const ForceArgs &A, int64_t s, int64_t bx, int by, i
     Acc7 hi[R], lo[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) { zero(p[r]); zero(hi[r]); zero(lo[r]); }
-    // two pair records per thread in flight (their loads are issued together),
-    // a fold after every kFoldPairs / 2 records
+    // two pair records per thread in flight (their loads are issued together), a fold
+    // after every kFoldPairs / 2 records (R = 2 runs on shares of up to kShortTiles
+    // tiles only, which one fold at the end covers: registers)
+    static_assert(kShortTiles / 2 <= kFoldPairs / 2, "one record per thread and two tiles");
     int cnt = 0;
-    for (int64_t pp = p0 + tid; pp < p1; pp += 2 * kThreads) {
-        const int64_t pq = pp + kThreads < p1 ? pp + kThreads : pp;
+    for (int pp = p0 + tid; pp < p1; pp += 2 * kThreads) {
+        const int pq = pp + kThreads < p1 ? pp + kThreads : pp;
         float4 a0, a1, a2, a3, a4, b0, b1, b2, b3, b4;
         {
             const float4 *q = A.j.p[pp].q;
@@ -375,32 +432,18 @@ __device__ void work_stream(const ForceArgs &A, int64_t s, int64_t bx, int by, i
                 pair_packed<true>(b0, b1, b2, b3, b4, ip[r], e2, p[r], 2 * pq == gi[r], 2 * pq + 1 == gi[r]);
         }
         cnt += 2;
-        if (cnt >= kFoldPairs / 2) {
+        if (R == 1 && cnt >= kFoldPairs / 2) {
             cnt = 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) fold(hi[r], lo[r], p[r]);
+            fold(hi[0], lo[0], p[0]);
         }
     }
-#pragma unroll
-    for (int r = 0; r < R; ++r) fold(hi[r], lo[r], p[r]);
-    // fixed-order reduction: lanes (xor tree of two-sums), then warps in ascending order
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        ds_group_reduce7<32>(hi[r], lo[r]);
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 7; ++c) sm->red[warp][r * 7 + c] = make_float2(acc_get(hi[r], c), acc_get(lo[r], c));
-        }
+        fold(hi[r], lo[r], p[r]);
+        cta_sum_red(hi[r], lo[r], &sm->red[warp][7 * r]);
     }
     __syncthreads();
-    if (tid < R * 7) {
-        float h = sm->red[0][tid].x, l = sm->red[0][tid].y;
-#pragma unroll
-        for (int wv = 1; wv < kThreads / 32; ++wv) ds_add(h, l, sm->red[wv][tid].x, sm->red[wv][tid].y);
-        int r = tid / 7, c = tid % 7;
-        int64_t ii = bx * R + r;
-        if (ii < s) part2(A, ii, by, S)[c] = make_float2(h, l);
-    }
+    cta_sum_out<R>(A, w, sm);
     __syncthreads();
 }
 
@@ -418,13 +461,13 @@ __device__ __forceinline__ void issue_ring(const ForceArgs &A, Smem *sm, int64_t
     bulk_g2s(sm->ring[st], A.j.p + tile * kPT, bytes, &sm->bar[st]);
 }
 
-__device__ void work_stream_tma(const ForceArgs &A, int64_t s, int64_t bx, int by, int S, Smem *sm, uint32_t &git)
+__device__ void work_stream_tma(const ForceArgs &A, int64_t w, Smem *sm, uint32_t &git)
 {
     static_assert(kThreads == 2 * kPT, "each half of the CTA takes one tile");
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t tper = qdiv(A.tile_hi - A.tile_lo + S - 1, S);
-    const int64_t t0 = A.tile_lo + (int64_t)by * tper;
-    const int64_t t1 = t0 + tper < A.tile_hi ? t0 + tper : A.tile_hi;
+    const int tid = threadIdx.x;
+    int64_t bx, t0, t1;
+    stream_item(A, w, sm, bx, t0, t1);
+    const int64_t s = sm->s;
     const int64_t nt = t1 > t0 ? t1 - t0 : 0;
     if (tid == 0) {
         const int64_t pro = nt < kRing ? nt : kRing;
@@ -478,141 +521,408 @@ __device__ void work_stream_tma(const ForceArgs &A, int64_t s, int64_t bx, int b
     }
     git += (uint32_t)nt;
     fold(hi, lo, p);
-    // fixed-order reduction: lanes (xor tree of two-sums), then warps in ascending order
-    ds_group_reduce7<32>(hi, lo);
+    cta_sum_red(hi, lo, sm->red[tid >> 5]);
+    __syncthreads();
+    cta_sum_out<1>(A, w, sm);
+    __syncthreads();
+}
+
+// ----------------------------------------------------------- column kernel
+// Variants 1 to 4: blocks of more than a few particles (see short_items).
+//
+// A variant's FP32 partial sums run over 32 pair records each before they are folded
+// into the two-sum accumulators. Over the records of a share (the table's split S gives
+// every i-particle S shares of tper tiles) they form columns: with stride st (256, 32, 8
+// or 1 records for variants 1, 2, 3, 4), 32 st consecutive records are a 32 x st matrix,
+// row by row, and each column is one FP32 sum (for st = 1 a column is 32 consecutive
+// records). The order of the columns is free: it only enters the two-sums. So
+//   * a unit is up to kUnitRec records, as many whole columns of one matrix as fit; its
+//     rows are copied into shared memory by the bulk engine, kSlots units in flight;
+//   * a CTA holds an i-block of I = 256 / TJ particles, TJ threads to each on different
+//     columns. Neighbouring lanes hold different particles and the same column, so a
+//     record is one broadcast for a warp (lanes on four columns would take twice the
+//     shared-memory wavefronts and hold the loop up). No record is read from L2 more
+//     than once per i-block, and the TJ threads' sums meet once per i-block;
+//   * the (i-block, unit) pairs are laid out in one line and cut into equal runs, one
+//     per CTA, whatever s, n and S. A run may end one i-block and begin the next; the
+//     last CTA of an i-block adds its partials in CTA order.
+//
+// What bounds it: the operand reads of the pair arithmetic (the register file delivers
+// two 32-bit operands per lane and clock; a packed FMA with three distinct operands
+// takes 1.45x one with two, so a record costs ~90 clocks a warp where the FP32 pipe
+// alone would take 76), i.e. 8.9e11 pairs/s. Measured against items of (i-block, share)
+// with 1, 2, 8, 32 or 256 particles, dealt out in advance (us a call): N = 65536: s = 480
+// 71.3 -> 59.4, 1024 150 -> 100, 5000 862 -> 417, N 5850 -> 5010; N = 200000, s = 700 298
+// -> 196; N = 300007: s = 33 49 -> 31, 61 47.9 -> 40.9; N = 2^20: s = 64 115 -> 108, 1024
+// 1424 -> 1300; N = s = 131072 20480 -> 19990 (94 clocks a record).
+
+__device__ __forceinline__ int variant_lgst(int v) { return v == 1 ? 8 : (v == 2 ? 5 : (v == 3 ? 3 : 0)); }
+// tiles per matrix (log2)
+__device__ __forceinline__ int matrix_lg(int lgst) { return lgst == 8 ? 6 : (lgst == 5 ? 3 : 1); }
+
+// Threads per particle (log2, at most 5). Wide i-blocks read each record for more
+// particles; narrower ones leave fewer lanes without a particle (at most 1 in 16
+// here), give every i-block fewer partials (the last CTA adds I G / nib of 64 bytes
+// each, kept near kColSum bytes), and cut the work finer (kColUnits units per CTA for
+// equal runs; not below 32 particles for this).
+constexpr int64_t kColSum = 128 << 10;
+constexpr int64_t kColUnits = 16;
+__device__ __forceinline__ int cols_lgtj(int64_t s, int64_t grid, int64_t upi)
+{
+    int lg = 0;
+    for (; lg < 5; ++lg) {
+        const int64_t I = kThreads >> lg, nib = (s + I - 1) >> (8 - lg);
+        if (16 * (nib * I - s) <= s && I * grid * 64 <= kColSum * nib && (lg >= 3 || nib * upi >= kColUnits * grid))
+            break;
+    }
+    return lg;
+}
+
+// Partial slots per particle: an i-block meets at most ceil(G / nib) + 1 runs.
+__device__ __forceinline__ int cols_slots(int64_t G, int64_t nib) { return (int)(G <= nib ? 2 : qdiv(G + nib - 1, nib) + 1); }
+
+// (few divisions: they are the longest part of the start of a small launch)
+__device__ __forceinline__ ColPlan cols_plan(const ForceArgs &A, int variant, int64_t s, int S)
+{
+    ColPlan P;
+    const int64_t T = A.tile_hi - A.tile_lo, grid = gridDim.x, me = blockIdx.x;
+    P.tper = S == 1 ? T : qdiv(T + S - 1, S);
+    const int64_t shares = S == 1 ? 1 : qdiv(T + P.tper - 1, P.tper);
+    P.lgst = variant_lgst(variant);
+    // rows of a share's first matrix, columns per unit
+    const int lgmt = matrix_lg(P.lgst);
+    const int nt = P.tper < (1 << lgmt) ? (int)P.tper : 1 << lgmt;
+    const int rows = P.lgst == 8 ? (nt + 1) / 2 : (P.lgst == 5 ? 4 * nt : (P.lgst == 3 ? 16 * nt : 32));
+    const int top = P.lgst == 8 ? 7 : (P.lgst == 5 ? 5 : 3);
+    P.lgcw = rows <= 1 ? 8 : 8 - (32 - __clz(rows - 1));   // floor(log2(kUnitRec / rows))
+    if (P.lgcw > top) P.lgcw = top;
+    P.ups = (int)((P.tper + (1 << lgmt) - 1) >> lgmt) << (P.lgst > P.lgcw ? P.lgst - P.lgcw : 0);
+    P.upi = shares * P.ups;
+    P.lgtj = cols_lgtj(s, grid, P.upi);
+    P.nib = (s + (kThreads >> P.lgtj) - 1) >> (8 - P.lgtj);
+    P.slots = cols_slots(grid, P.nib);
+    // never more partials than there is room for (the no-allocation entry point has room
+    // for few): more, smaller i-blocks; without any room, whole i-blocks to a CTA
+    while (s * P.slots * kPartStride > A.part_cap && P.lgtj < 5) {
+        ++P.lgtj;
+        P.nib = (s + (kThreads >> P.lgtj) - 1) >> (8 - P.lgtj);
+        P.slots = cols_slots(grid, P.nib);
+    }
+    const bool whole = s * P.slots * kPartStride > A.part_cap;
+    if (whole) {
+        P.lgtj = 3;
+        P.nib = (s + (kThreads >> P.lgtj) - 1) >> (8 - P.lgtj);
+    }
+    P.U = P.nib * P.upi;
+    const int64_t line = whole ? P.nib : P.U, step = whole ? P.upi : 1;
+    P.G = grid < line ? grid : line;
+    P.u0 = P.u1 = P.b0 = 0;
+    if (me < P.G) {
+        P.u0 = qdiv(line * me, P.G) * step;
+        P.u1 = qdiv(line * (me + 1), P.G) * step;
+        P.b0 = qdiv(P.u0, P.upi);
+    }
+    P.whole = whole ? 1 : 0;
+    return P;
+}
+
+// Where unit u of an i-block lies: record `rec` is row 0 of its first column, `rows`
+// rows of `cols` columns, 2^lgst records apart (st = 1: `cols` columns of 32
+// consecutive records).
+struct Unit {
+    int64_t rec;
+    int rows, cols;
+};
+__device__ __forceinline__ Unit unit_at(const ForceArgs &A, const ColPlan &P, int64_t u)
+{
+    const int64_t sh = P.upi == P.ups ? 0 : qdiv(u, P.ups);
+    const int v = (int)(u - sh * P.ups);
+    const int64_t t0 = A.tile_lo + sh * P.tper;
+    const int64_t t1 = t0 + P.tper < A.tile_hi ? t0 + P.tper : A.tile_hi;
+    const int lgch = P.lgst > P.lgcw ? P.lgst - P.lgcw : 0;   // column chunks per matrix
+    const int m = v >> lgch, c0 = (v - (m << lgch)) << P.lgcw;
+    const int lgmt = matrix_lg(P.lgst);
+    const int64_t ts = t0 + ((int64_t)m << lgmt);
+    int nt = t1 - ts < (1 << lgmt) ? (int)(t1 - ts) : 1 << lgmt;
+    if (nt < 0) nt = 0;
+    Unit q;
+    q.rec = ts * kPT + c0;
+    q.cols = P.lgst == 0 ? 4 * nt : 1 << P.lgcw;
+    q.rows = P.lgst == 8 ? (c0 >= 128 ? nt / 2 : (nt + 1) / 2) : (P.lgst == 5 ? 4 * nt : (P.lgst == 3 ? 16 * nt : 32));
+    return q;
+}
+
+// The unit, column and row of record r of the range (unit -1: r is outside the range).
+__device__ __forceinline__ int64_t unit_of(const ForceArgs &A, const ColPlan &P, int64_t r, int &col, int &row)
+{
+    col = row = 0;
+    const int64_t tile = (r >> 7) - A.tile_lo;
+    if (tile < 0 || r >= A.tile_hi * kPT) return -1;
+    const int64_t sh = P.upi == P.ups ? 0 : qdiv(tile, P.tper);
+    const int64_t rs = r - (A.tile_lo + sh * P.tper) * kPT;   // record within the share
+    const int lgm = 7 + matrix_lg(P.lgst);                    // records per matrix
+    const int64_t m = rs >> lgm;
+    const int rm = (int)(rs - (m << lgm));
+    if (P.lgst == 0) {
+        col = rm >> 5;
+        row = rm & 31;
+        return sh * P.ups + m;
+    }
+    const int c = rm & ((1 << P.lgst) - 1);
+    row = rm >> P.lgst;
+    col = c & ((1 << P.lgcw) - 1);
+    return sh * P.ups + (m << (P.lgst - P.lgcw)) + (c >> P.lgcw);
+}
+
+// Copies unit u into its slot (called by one warp): one copy where the unit's records
+// are consecutive, else one per row.
+__device__ __forceinline__ void unit_issue(const ForceArgs &A, Smem *sm, const ColPlan &P, int64_t u, int slot)
+{
+    const int lane = threadIdx.x & 31;
+    const Unit q = unit_at(A, P, u);
+    const uint32_t row = (uint32_t)sizeof(JPair) << P.lgcw;
+    const uint32_t all = P.lgst == 0 ? (uint32_t)q.cols * 32u * (uint32_t)sizeof(JPair) : (uint32_t)q.rows * row;
     if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) sm->red[warp][c] = make_float2(acc_get(hi, c), acc_get(lo, c));
+        sm->info[slot] = make_int2(q.rows, q.cols);   // read by the warps after the slot's barrier
+        mbar_arrive_expect_tx(&sm->bar[slot], all);
     }
-    __syncthreads();
-    if (tid < 7) {
-        float h = sm->red[0][tid].x, l = sm->red[0][tid].y;
-#pragma unroll
-        for (int wv = 1; wv < kThreads / 32; ++wv) ds_add(h, l, sm->red[wv][tid].x, sm->red[wv][tid].y);
-        if (bx < s) part2(A, bx, by, S)[tid] = make_float2(h, l);
+    __syncwarp();
+    if (P.lgst <= 3) {
+        if (lane == 0 && all) bulk_g2s(sm->unit[slot], A.j.p + q.rec, all, &sm->bar[slot]);
+    } else if (lane < q.rows) {
+        bulk_g2s(sm->unit[slot] + lane * row, A.j.p + q.rec + ((int64_t)lane << P.lgst), row, &sm->bar[slot]);
     }
-    __syncthreads();
 }
 
-// ----------------------------------------------------------- tiled variant
-// TI = kThreads / TJ thread groups, each holding R i-particles; the TJ threads
-// of a group take interleaved pair records of each shared-memory tile.
-template <int R, int TJ, bool MASK>
-__device__ __forceinline__ void sweep_tile(const Smem *sm, int st, int tj, int64_t j0, const IPk *ip,
-                                           const int32_t *gi, float2 e2, AccPk *p, Acc7 *hi, Acc7 *lo)
+// One column: rows records of hop bytes from src (ROWS, HOP: the usual ones, known to the
+// compiler). self: the row holding the i-particle itself, in lane b of the record if
+// odd; -1: none.
+template <bool MASK, int ROWS, int HOP>
+__device__ __forceinline__ void sweep_column(const unsigned char *src, int rows, int hop, int self, bool odd,
+                                             const IPk &ip, float2 e2, AccPk &p)
 {
-    constexpr int PPT = kPT / TJ;                           // pair records per thread per tile
-    constexpr int FP = kFoldPairs / 2;                      // records per fold
-    constexpr int CH = PPT < FP ? PPT : FP;
-    const JPair *T = sm->tile[st];
-#pragma unroll 1
-    for (int c0 = 0; c0 < PPT; c0 += CH) {
+    if (ROWS) rows = ROWS;
+    if (HOP) hop = HOP;
 #pragma unroll 4
-        for (int u = 0; u < CH; ++u) {
-            const int pp = tj + (c0 + u) * TJ;
-            const float4 q0 = T[pp].q[0], q1 = T[pp].q[1], q2 = T[pp].q[2], q3 = T[pp].q[3], q4 = T[pp].q[4];
-            const int64_t ja = j0 + 2 * pp;
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                pair_packed<MASK>(q0, q1, q2, q3, q4, ip[r], e2, p[r], MASK && ja == gi[r], MASK && ja + 1 == gi[r]);
-        }
-        if (PPT >= FP) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) fold(hi[r], lo[r], p[r]);
-        }
+    for (int m = 0; m < rows; ++m) {
+        const float4 *Q = reinterpret_cast<const float4 *>(src + m * hop);
+        const float4 q0 = Q[0], q1 = Q[1], q2 = Q[2], q3 = Q[3], q4 = Q[4];
+        pair_packed<MASK>(q0, q1, q2, q3, q4, ip, e2, p, MASK && m == self && !odd, MASK && m == self && odd);
     }
 }
 
-__device__ __forceinline__ void issue_tile(const ForceArgs &A, Smem *sm, int64_t tile, int st)
+// The sums of i-block b: every thread's (hi, lo), first over the lanes of a warp that
+// hold the same particle (I < 32), then over the warps through shared memory, into the
+// CTA's partial slot or, with n == 1 (no other CTA has a part), the results.
+__device__ __forceinline__ void cols_out(const ForceArgs &A, int64_t s, int64_t ib0, int lgi, int n, int slot, Acc7 &hi,
+                                         Acc7 &lo, Smem *sm)
 {
-    constexpr uint32_t bytes = kPT * sizeof(JPair);
-    mbar_arrive_expect_tx(&sm->bar[st], bytes);
-    bulk_g2s(sm->tile[st], A.j.p + tile * kPT, bytes, &sm->bar[st]);
-}
-
-template <int R, int TJ>
-__device__ void work_tile(const ForceArgs &A, int64_t s, int64_t bx, int by, int S, Smem *sm, uint32_t &git)
-{
-    constexpr int TI = kThreads / TJ;
-    constexpr int I = TI * R;
-    constexpr int PPT = kPT / TJ;
-    constexpr int kFoldTiles = PPT >= kFoldPairs / 2 ? 0 : (kFoldPairs / 2) / PPT;   // 0: folded inside the sweep
-    static_assert(TJ <= 32 && (32 % TJ) == 0, "TJ must divide a warp");
-    const int tid = threadIdx.x, tj = tid % TJ, ti = tid / TJ;
-    const int64_t tper = qdiv(A.tile_hi - A.tile_lo + S - 1, S);
-    const int64_t t0 = A.tile_lo + (int64_t)by * tper;
-    const int64_t t1 = t0 + tper < A.tile_hi ? t0 + tper : A.tile_hi;
-    const int64_t nt = t1 > t0 ? t1 - t0 : 0;
-    // the first tiles are in flight before the i-particle loads
-    if (tid == 0) {
-        const int64_t pro = nt < kStages - 1 ? nt : kStages - 1;
-        for (int64_t q = 0; q < pro; ++q) issue_tile(A, sm, t0 + q, (int)((git + q) % kStages));
+    const int tid = threadIdx.x;
+    for (int off = 16; off >= (1 << lgi); off >>= 1) {
+        Acc7 h2, l2;
+        h2.ax = __shfl_xor_sync(0xffffffffu, hi.ax, off); l2.ax = __shfl_xor_sync(0xffffffffu, lo.ax, off);
+        h2.ay = __shfl_xor_sync(0xffffffffu, hi.ay, off); l2.ay = __shfl_xor_sync(0xffffffffu, lo.ay, off);
+        h2.az = __shfl_xor_sync(0xffffffffu, hi.az, off); l2.az = __shfl_xor_sync(0xffffffffu, lo.az, off);
+        h2.kx = __shfl_xor_sync(0xffffffffu, hi.kx, off); l2.kx = __shfl_xor_sync(0xffffffffu, lo.kx, off);
+        h2.ky = __shfl_xor_sync(0xffffffffu, hi.ky, off); l2.ky = __shfl_xor_sync(0xffffffffu, lo.ky, off);
+        h2.kz = __shfl_xor_sync(0xffffffffu, hi.kz, off); l2.kz = __shfl_xor_sync(0xffffffffu, lo.kz, off);
+        h2.ph = __shfl_xor_sync(0xffffffffu, hi.ph, off); l2.ph = __shfl_xor_sync(0xffffffffu, lo.ph, off);
+        ds_add(hi.ax, lo.ax, h2.ax, l2.ax);
+        ds_add(hi.ay, lo.ay, h2.ay, l2.ay);
+        ds_add(hi.az, lo.az, h2.az, l2.az);
+        ds_add(hi.kx, lo.kx, h2.kx, l2.kx);
+        ds_add(hi.ky, lo.ky, h2.ky, l2.ky);
+        ds_add(hi.kz, lo.kz, h2.kz, l2.kz);
+        ds_add(hi.ph, lo.ph, h2.ph, l2.ph);
     }
-
-    IPk ip[R];
-    int32_t gi[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        int64_t ii = bx * I + (int64_t)r * TI + ti;
-        gi[r] = idx_at(A, sm, ii < s ? ii : s - 1);
-        ip[r] = ipk_of(jrec_load(A.j.p, gi[r]));
-    }
-    const float2 e2 = make_float2(A.eps2f, A.eps2f);
-    // index range of this i-block (the active list ascends), for self-exclusion
-    const int64_t ib0 = bx * I;
-    const int64_t ib1 = (ib0 + I < s ? ib0 + I : s) - 1;
-    const int64_t imin = idx_at(A, sm, ib0), imax = idx_at(A, sm, ib1);
-
-    AccPk p[R];
-    Acc7 hi[R], lo[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) { zero(p[r]); zero(hi[r]); zero(lo[r]); }
-    int fc = 0;
-    for (int64_t q = 0; q < nt; ++q) {
-        const uint32_t g = git + (uint32_t)q;
-        const int st = (int)(g % kStages);
-        if (tid == 0 && q + kStages - 1 < nt)
-            issue_tile(A, sm, t0 + q + kStages - 1, (int)((g + kStages - 1) % kStages));
-        if (!mbar_wait(&sm->bar[st], (g / kStages) & 1u, A.spin_limit)) sm->abort = 1;
-        const int64_t j0 = (t0 + q) * kJT;
-        if (j0 <= imax && j0 + kJT - 1 >= imin)
-            sweep_tile<R, TJ, true>(sm, st, tj, j0, ip, gi, e2, p, hi, lo);
+    for (int c = 0; c < 7; ++c) sm->sums[c][tid] = make_float2(acc_get(hi, c), acc_get(lo, c));
+    __syncthreads();
+    const int I = 1 << lgi, hop = I < 32 ? 32 : I, W = kThreads / hop;
+    for (int o = tid; o < 8 * I; o += kThreads) {
+        const int c = o & 7, i = o >> 3;
+        if (c == 7 || ib0 + i >= s) continue;
+        float h = sm->sums[c][i].x, l = sm->sums[c][i].y;
+        for (int w = 1; w < W; ++w) ds_add(h, l, sm->sums[c][i + w * hop].x, sm->sums[c][i + w * hop].y);
+        if (n == 1)
+            put_final(A, ib0 + i, c, (double)h + (double)l);
         else
-            sweep_tile<R, TJ, false>(sm, st, tj, j0, ip, gi, e2, p, hi, lo);
-        if (kFoldTiles > 0 && ++fc == kFoldTiles) {
-            fc = 0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) fold(hi[r], lo[r], p[r]);
+            part2(A, ib0 + i, slot, sm->plan.slots)[c] = make_float2(h, l);
+    }
+}
+
+// This CTA's run. False: a wait ran out.
+__device__ bool work_cols(const ForceArgs &A, int64_t s, Smem *sm)
+{
+    const ColPlan &P = sm->plan;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int lgtj = P.lgtj, lgi = 8 - lgtj, tj = tid >> lgi, ti = tid & ((1 << lgi) - 1);
+    const int lgnu = lgtj > P.lgcw ? lgtj - P.lgcw : 0;    // units side by side
+    const int cstep = lgnu ? 1 << P.lgcw : 1 << lgtj;      // a thread's columns: c0, c0 + cstep, ...
+    const int ncol = lgnu ? 1 : 1 << (P.lgcw - lgtj);      // of them per unit
+    const int c0 = tj & (cstep - 1);
+    const int mine = lgnu ? tj >> P.lgcw : 0;              // this thread's unit of a round
+    // slots are refilled one round behind, when all warps have most likely left them
+    // (rounds of more than half of the slots: at once)
+    const int ahead = kSlots - ((2 << lgnu) <= kSlots ? 1 << lgnu : 0);
+    const int hop = P.lgst == 0 ? (int)sizeof(JPair) : (int)sizeof(JPair) << P.lgcw;
+    const int chop = P.lgst == 0 ? 32 * (int)sizeof(JPair) : (int)sizeof(JPair);
+    const float2 e2 = make_float2(A.eps2f, A.eps2f);
+    volatile int *stop = &sm->abort;
+    const int64_t u0 = P.u0, u1 = P.u1;
+    int64_t b = P.b0;
+    int64_t ub = b * P.upi;         // first unit of i-block b
+    const int64_t place0 = u0 - ub; // unit v of the run is at place (place0 + v) mod upi of its i-block
+    if (warp < kSlots && u0 + warp < u1) unit_issue(A, sm, P, place0 + warp < P.upi ? place0 + warp : qmod(place0 + warp, P.upi), warp);
+    uint32_t used = 0;              // units of the run this warp is done with
+    bool ok = true;
+    for (int64_t u = u0; u < u1; ++b, ub += P.upi) {
+        const int64_t ue = ub + P.upi < u1 ? ub + P.upi : u1;
+        const int64_t ib0 = b << lgi, ii = ib0 + ti;
+        const int32_t gi = idx_at(A, sm, ii < s ? ii : s - 1);
+        const IPk ip = ipk_of(jrec_load(A.j.p, gi));
+        int scol, srow;
+        const int64_t su = unit_of(A, P, gi >> 1, scol, srow) + ub;   // the i-particle's own place
+        if (tid == 0) {
+            // the runs that meet this i-block
+            const int64_t first = qdiv((ub + 1) * P.G - 1, P.U);
+            sm->plan.part_n = P.whole ? 1 : (int)(qdiv((ub + P.upi) * P.G - 1, P.U) - first) + 1;
+            sm->plan.part_slot = (int)(blockIdx.x - first);
         }
-        __syncthreads();
-        if (sm->abort) {
-            // a wait ran out: drain what this CTA still has in flight (bounded), then stop
-            if (tid == 0) {
-                for (int64_t qq = q + 1; qq < nt && qq < q + kStages; ++qq) {
-                    const uint32_t gg = git + (uint32_t)qq;
-                    (void)mbar_wait(&sm->bar[gg % kStages], (gg / kStages) & 1u, A.spin_limit);
+        AccPk p;
+        Acc7 hi, lo;
+        zero(p);
+        zero(hi);
+        zero(lo);
+        while (u < ue) {
+            // a round: 2^lgnu units (the last one of an i-block or run may have fewer)
+            const int cnt = ue - u < (1 << lgnu) ? (int)(ue - u) : 1 << lgnu;
+            const bool have = mine < cnt;
+            const uint32_t v = used + (uint32_t)(have ? mine : 0);
+            const int sl = (int)(v % kSlots);
+            ok = mbar_wait(&sm->bar[sl], (v / kSlots) & 1u, A.spin_limit);
+            if (__all_sync(0xffffffffu, ok)) {
+                const int2 q = sm->info[sl];
+                const bool self = have && u + mine == su;
+                const unsigned char *src = sm->unit[sl] + c0 * chop;
+                const bool plain = have && !self && q.x == 32 && q.y >= cstep * ncol;
+                if (__all_sync(0xffffffffu, plain) && (hop == (int)sizeof(JPair) || hop == 8 * (int)sizeof(JPair))) {
+                    for (int it = 0; it < ncol; ++it, src += cstep * chop) {
+                        if (hop == (int)sizeof(JPair))
+                            sweep_column<false, 32, (int)sizeof(JPair)>(src, 32, hop, -1, false, ip, e2, p);
+                        else
+                            sweep_column<false, 32, 8 * (int)sizeof(JPair)>(src, 32, hop, -1, false, ip, e2, p);
+                        fold(hi, lo, p);
+                    }
+                } else {
+                    for (int it = 0; it < ncol; ++it, src += cstep * chop) {
+                        const int c = c0 + it * cstep;
+                        const int rows = have && c < q.y ? q.x : 0;
+                        const bool here = self && c == scol;
+                        if (__any_sync(0xffffffffu, here))
+                            sweep_column<true, 0, 0>(src, rows, hop, here ? srow : -1, gi & 1, ip, e2, p);
+                        else
+                            sweep_column<false, 0, 0>(src, rows, hop, -1, false, ip, e2, p);
+                        fold(hi, lo, p);
+                    }
                 }
             }
-            git += (uint32_t)nt;
-            return;
+            if (!__all_sync(0xffffffffu, ok)) *stop = 1;
+            if (*stop) break;
+            __syncwarp();   // this warp has read the round's units
+            if (lane < cnt) mbar_arrive(&sm->empty[(used + lane) % kSlots]);
+            // the warps take turns at refilling
+            for (int q = 0; q < cnt; ++q) {
+                const uint32_t w = used + (uint32_t)(ahead + q);   // unit to copy
+                if (w < kSlots || (w & (kThreads / 32 - 1)) != (uint32_t)warp || u0 + w >= u1) continue;
+                ok = mbar_wait(&sm->empty[w % kSlots], (w / kSlots - 1) & 1u, A.spin_limit);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    *stop = 1;
+                    break;
+                }
+                unit_issue(A, sm, P, qmod(place0 + w, P.upi), (int)(w % kSlots));
+            }
+            used += cnt;
+            u += cnt;
+        }
+        if (__syncthreads_or(!ok || *stop)) {
+            // a wait ran out somewhere in the CTA: drain what may be in flight (bounded), stop
+            if (tid == 0)
+                for (uint32_t q = 0; q < 2 * kSlots; ++q) {
+                    const uint32_t w = used + q < kSlots ? q : used + q - kSlots;
+                    if (u0 + w < u1) (void)mbar_wait(&sm->bar[w % kSlots], (w / kSlots) & 1u, A.spin_limit);
+                }
+            return false;
+        }
+        const int n = sm->plan.part_n;
+        cols_out(A, s, ib0, lgi, n, sm->plan.part_slot, hi, lo, sm);
+        if (n > 1) {
+            const int64_t ib1 = ib0 + (1 << lgi);
+            finish_block(A, b, ib0, ib1 < s ? ib1 : s, P.slots, n, sm);
         }
     }
-    git += (uint32_t)nt;
-#pragma unroll
-    for (int r = 0; r < R; ++r) fold(hi[r], lo[r], p[r]);
+    return true;
+}
 
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (TJ > 1) ds_group_reduce7<TJ>(hi[r], lo[r]);
-        const int64_t ii = bx * I + (int64_t)r * TI + ti;
-        if (tj == 0 && ii < s) write_part(A, ii, by, S, hi[r], lo[r]);
+// --------------------------------------------------- short shares, variant 2
+// Eight particles per CTA, one per warp, a lane per column (stride 32): an item's
+// tiles, up to kShortRing at once, are copied into shared memory in one go. For blocks
+// so small that one item per CTA covers them: no plan, no ring, no meeting of warps.
+constexpr int kShortRing = (int)(sizeof(Smem::unit) / (kPT * sizeof(JPair)));
+static_assert(kShortRing == 8, "the fold falls on whole turns (32 rows are 8 tiles)");
+
+__device__ void work_tile32(const ForceArgs &A, int64_t w, Smem *sm, uint32_t &git)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t bx, t0, t1;
+    stream_item(A, w, sm, bx, t0, t1);
+    const int64_t ii = bx * 8 + warp;
+    const int32_t gi = idx_at(A, sm, ii < sm->s ? ii : sm->s - 1);
+    IPk ip;
+    AccPk p;
+    Acc7 hi, lo;
+    zero(p);
+    zero(hi);
+    zero(lo);
+    const float2 e2 = make_float2(A.eps2f, A.eps2f);
+    const JPair *rec = reinterpret_cast<const JPair *>(sm->unit[0]);
+    for (int64_t t = t0; t < t1; t += kShortRing) {
+        const int nt = t1 - t < kShortRing ? (int)(t1 - t) : kShortRing;
+        if (tid == 0) {
+            constexpr uint32_t bytes = kPT * sizeof(JPair);
+            mbar_arrive_expect_tx(&sm->bar[0], (uint32_t)nt * bytes);
+            for (int q = 0; q < nt; ++q)
+                bulk_g2s(sm->unit[0] + q * bytes, A.j.p + (t + q) * kPT, bytes, &sm->bar[0]);
+        }
+        if (t == t0) ip = ipk_of(jrec_load(A.j.p, gi));
+        // the particle's own row, if its record is in this lane's column
+        const int64_t rel = (gi >> 1) - t * kPT;
+        const int self = rel >= 0 && rel < nt * kPT && ((int)rel & 31) == lane ? (int)rel >> 5 : -1;
+        if (!mbar_wait(&sm->bar[0], git & 1u, A.spin_limit)) sm->abort = 1;
+        ++git;
+        if (__syncthreads_or(sm->abort)) return;   // (the wait that failed was the drain)
+#pragma unroll 4
+        for (int m = 0; m < 4 * nt; ++m) {
+            const float4 *Q = rec[32 * m + lane].q;
+            pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, m == self && !(gi & 1), m == self && (gi & 1));
+        }
+        fold(hi, lo, p);
+        __syncthreads();   // the tiles have been read
+    }
+    float h, l;
+    const int c = ds_scatter_reduce<32>(hi, lo, h, l);
+    if ((lane & 3) == 0 && c < 7 && ii < sm->s) {
+        if (sm->split == 1)
+            put_final(A, ii, c, (double)h + (double)l);
+        else
+            part2(A, ii, (int)(w - bx * sm->split), sm->split)[c] = make_float2(h, l);
     }
 }
 
 // -------------------------------------------------------------- variants
 
-// 0: stream R=1 (I=1)      1: stream R=2 (I=2)      2: tile R=1 TJ=32 (I=8)
-// 3: tile R=1 TJ=8 (I=32)  4: tile R=1 TJ=1 (I=256) 5: TMA stream R=1 (I=1)
+// 0: stream (one particle per CTA)   5: TMA stream (the same sums)
+// 1, 2, 3, 4: columns with stride 256, 32, 8, 1
 // 6: resident share (cluster launch; the split factor is unused)
 constexpr int kMixedFallback = kMixedFallbackId;   // the variant of an out-of-range table entry
 constexpr int kShareVariant = kShareVariantId;
@@ -835,6 +1145,16 @@ __device__ __noinline__ void share_force(const ForceArgs &A, int64_t s, Smem *sm
     if (!ok && nrec > 0 && tid == 0) (void)mbar_wait(&sm->bar[0], 0, A.spin_limit);   // drain before exit
 }
 
+// Variants 1 and 2 where one item (two or eight particles, one share) per CTA covers the
+// block and the shares are short: such a launch is a chain of latencies, and the
+// columns' plan, ring and meeting of warps lengthen it (us under the profiler, items
+// against columns: N = 10^5, s = 2 10.4 / 17.2, s = 24 13.2 / 15.9; N = 65536, s = 20 12.4 /
+// 15.5). Longer or more items: the columns (N = 65536, s = 100 25.9 against 31.9).
+__device__ __forceinline__ bool short_items(int variant, int64_t T, int S, int64_t items)
+{
+    return variant <= 2 && items <= gridDim.x && T <= kShortTiles * (int64_t)S;
+}
+
 // SHARE: the instantiation with the resident-share variant (launched as clusters
 // with kSmemShare bytes); without it the kernel has no cluster code and the
 // plain shared-memory size.
@@ -852,6 +1172,7 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
     const int32_t ipre = tid < A.idx_cap ? A.idx[tid] : 0;
     if (tid == 0) {
         for (int st = 0; st < kRing; ++st) mbar_init(&sm->bar[st], 1);
+        for (int st = 0; st < kSlots; ++st) mbar_init(&sm->empty[st], kThreads / 32);
         mbar_init(&sm->inject_bar, 1);
         fence_mbar_init();
         sm->abort = 0;
@@ -902,26 +1223,40 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
     }
     S = clamp_split(S, A.tile_hi - A.tile_lo, s, A.part_cap);
     if (blockIdx.x == 0 && tid == 0) *A.split_used = S;
-    const int64_t I = mixed_I(variant);
-    const int64_t nib = qdiv(s + I - 1, I);
-    const int64_t W = nib * S;
+    const int64_t T = A.tile_hi - A.tile_lo;
+    const int lgi = variant == 1 ? 1 : (variant == 2 ? 3 : 0);
+    if (variant >= 1 && variant <= 4 && !short_items(variant, T, S, ((s + (1 << lgi) - 1) >> lgi) * S)) {
+        if (tid == 0) sm->plan = cols_plan(A, variant, s, S);
+        __syncthreads();
+        if (blockIdx.x < sm->plan.G && !work_cols(A, s, sm) && tid == 0) atomicOr(A.status, kStTimeout);
+        return;
+    }
+    // work items (i-block of 1, 2 or 8 particles, share)
+    if (tid == 0) {
+        sm->split = S;
+        sm->lgi = lgi;
+        sm->tper = S == 1 ? T : qdiv(T + S - 1, S);
+        sm->items = ((s + (1 << lgi) - 1) >> lgi) * S;
+    }
+    __syncthreads();
     uint32_t git = 0;
-    for (int64_t w = blockIdx.x; w < W; w += gridDim.x) {
-        const int64_t bx = qdiv(w, S);
-        const int by = (int)(w - bx * S);
-        switch (variant) {
-        case 0: work_stream<1>(A, s, bx, by, S, sm); break;
-        case 1: work_stream<2>(A, s, bx, by, S, sm); break;
-        case 2: work_tile<1, 32>(A, s, bx, by, S, sm, git); break;
-        case 3: work_tile<1, 8>(A, s, bx, by, S, sm, git); break;
-        case 5: work_stream_tma(A, s, bx, by, S, sm, git); break;
-        default: work_tile<1, 1>(A, s, bx, by, S, sm, git); break;
-        }
+    for (int64_t w = blockIdx.x; w < sm->items; w += gridDim.x) {
+        if (variant == 1)
+            work_stream<2>(A, w, sm);
+        else if (variant == 2)
+            work_tile32(A, w, sm, git);
+        else if (variant == 0)
+            work_stream<1>(A, w, sm);
+        else
+            work_stream_tma(A, w, sm, git);
         if (sm->abort) {
             if (tid == 0) atomicOr(A.status, kStTimeout);
             return;
         }
-        finish_item(A, s, bx, S, I, sm);
+        if (sm->split > 1) {
+            const int64_t bx = qdiv(w, sm->split), i0 = bx << sm->lgi, i1 = (bx + 1) << sm->lgi;
+            finish_block(A, bx, i0, i1 < sm->s ? i1 : sm->s, sm->split, sm->split, sm);
+        }
     }
 }
 
@@ -1331,11 +1666,10 @@ void default_tuning(int precision, int64_t n, int64_t s, int num_sms, int ctas_p
         // the j-records fit the resident shares of a cluster: no split partials in L2
         v = kShareVariant;
     } else if (n <= 65536) {
-        // j-records stay in L2 and are cheap to re-read: stream variants (every
-        // thread of a CTA on the same 1 or 2 i-particles) win while blocks are small
+        // j-records stay in L2 and are cheap to re-read: wide columns while blocks are small
         v = s <= (n <= 32768 ? 64 : 16) ? 0 : s <= 1024 ? 1 : s <= 1536 ? 2 : s <= 12288 ? 3 : 4;
     } else {
-        // large N: re-reading all j per i-particle costs more than it hides
+        // large N: narrower columns, fewer shares
         v = s <= 1 ? 0 : s <= 4 ? 1 : s <= 32 ? 2 : s <= 512 ? 3 : 4;
     }
     const int64_t I = mixed_I(v);

@@ -78,7 +78,7 @@ struct ForceArgs {
     double *part;         // split partials [s][split][8] (mixed: float2 (hi, lo) pairs)
     int64_t part_cap;     // capacity of part in 8-byte words
     double *fin;          // final sums [s][8]: ax ay az kx ky kz phi pad
-    int32_t *tickets;     // per i-block arrival counters (zero between launches)
+    int32_t *tickets;     // arrival counters of the i-blocks (zero between launches)
     int32_t *split_used;  // written by the kernel: split factor of this launch
     const Tuning *tune;   // device tuning table
     int32_t force_variant;  // >= 0: ignore the table (autotuner, tests)
@@ -105,10 +105,10 @@ cudaError_t launch_perturbers(const PertArgs &p, cudaStream_t st);
 
 // Variant catalogue. Mixed: 0..kMixedVariants-1; FP64: 0..kF64Variants-1.
 constexpr int kMixedVariants = 7;
-constexpr int kMixedFallbackId = 4;   // tiled, one particle per thread: takes any size
+constexpr int kMixedFallbackId = 4;   // columns of 32 consecutive records: takes any size
 constexpr int kShareVariantId = 6;    // resident j-share in 8-CTA clusters
 constexpr int kF64Variants = 2;
-int mixed_variant_I(int v);           // i-particles per work item
+int mixed_variant_I(int v);           // i-particles the table's split counts as one i-block
 const char *mixed_variant_name(int v);
 int f64_variant_I(int v);
 const char *f64_variant_name(int v);

@@ -158,6 +158,76 @@ __device__ __forceinline__ void ds_group_reduce7(Acc7 &hi, Acc7 &lo)
     }
 }
 
+// The sums of the seven components over a group of G lanes, spread over the group:
+// every step halves the components a lane carries as well as the lanes they are spread
+// over (4 + 2 + 1 two-sum additions for G = 8 where the butterfly above takes 21). A
+// lane ends with max(1, 8 / G) components, the first of which is returned (component
+// 7 is padding); for G > 8 the lanes of each run of G / 8 hold the same sum.
+template <int G, int N>
+__device__ __forceinline__ int ds_scatter_reduce(const Acc7 &hi, const Acc7 &lo, float (&oh)[N], float (&ol)[N])
+{
+    static_assert(N == (G >= 8 ? 1 : 8 / G), "components per lane");
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    float h[8] = {hi.ax, hi.ay, hi.az, hi.kx, hi.ky, hi.kz, hi.ph, 0.f};
+    float l[8] = {lo.ax, lo.ay, lo.az, lo.kx, lo.ky, lo.kz, lo.ph, 0.f};
+    int first = 0;
+    if (G >= 2) {
+        const bool up = lane & (G / 2);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float sh = up ? h[c] : h[c + 4], sl = up ? l[c] : l[c + 4];
+            if (up) {
+                h[c] = h[c + 4];
+                l[c] = l[c + 4];
+            }
+            ds_add(h[c], l[c], __shfl_xor_sync(full, sh, G / 2), __shfl_xor_sync(full, sl, G / 2));
+        }
+        first = up ? 4 : 0;
+    }
+    if (G >= 4) {
+        const bool up = lane & (G / 4);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float sh = up ? h[c] : h[c + 2], sl = up ? l[c] : l[c + 2];
+            if (up) {
+                h[c] = h[c + 2];
+                l[c] = l[c + 2];
+            }
+            ds_add(h[c], l[c], __shfl_xor_sync(full, sh, G / 4), __shfl_xor_sync(full, sl, G / 4));
+        }
+        first += up ? 2 : 0;
+    }
+    if (G >= 8) {
+        const bool up = lane & (G / 8);
+        const float sh = up ? h[0] : h[1], sl = up ? l[0] : l[1];
+        if (up) {
+            h[0] = h[1];
+            l[0] = l[1];
+        }
+        ds_add(h[0], l[0], __shfl_xor_sync(full, sh, G / 8), __shfl_xor_sync(full, sl, G / 8));
+        first += up ? 1 : 0;
+    }
+#pragma unroll
+    for (int off = G / 16; off >= 1; off >>= 1)
+        ds_add(h[0], l[0], __shfl_xor_sync(full, h[0], off), __shfl_xor_sync(full, l[0], off));
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        oh[q] = h[q];
+        ol[q] = l[q];
+    }
+    return first;
+}
+template <int G>
+__device__ __forceinline__ int ds_scatter_reduce(const Acc7 &hi, const Acc7 &lo, float &oh, float &ol)
+{
+    float h[1], l[1];
+    const int c = ds_scatter_reduce<G, 1>(hi, lo, h, l);
+    oh = h[0];
+    ol = l[0];
+    return c;
+}
+
 __device__ __forceinline__ float acc_get(const Acc7 &q, int c)
 {
     switch (c) {
