@@ -14,22 +14,23 @@
 // CTA r owns the particles [r c, (r + 1) c) (c = chunk). Per step it
 //   1. finds its chunk's members of the block (keys t + dt equal to the block
 //      time; ascending) and the smallest other key; pushes its member count into
-//      every CTA's shared memory;
+//      every CTA's shared memory (one warp);
 //   2. predicts its members to the block time (the double-single predictor of
-//      the full path, same bits) and pushes their records to every CTA;
+//      the full path, same bits) and pushes their records to every CTA (the same
+//      warp), while the other warps predict the whole chunk into pair records in
+//      shared memory;
 //   -- cluster barrier: every CTA knows every chunk's count, hence the block
 //      size s and each chunk's offset; if the block is too large for the engine
 //      (s > s_max, or more than kEngCap members in one chunk), past t_end, or
 //      the step budget is used up, every CTA stops here, leaving the block time
 //      for the full path;
-//   3. predicts its whole chunk into pair records in shared memory, orders the
-//      s members it received, and sums their forces over its own chunk only
+//   3. orders the s members it received and sums their forces over its own chunk only
 //      (packed f32x2 pair arithmetic, two-sum folds and reductions: the force
 //      kernel's arithmetic), pushing the (hi, lo) partial sums to each member's
 //      owner;
 //   -- cluster barrier;
 //   4. corrects its own members: four lanes per particle add the C partial sums
-//      in rank order (the paper's global sum of partial forces, in a fixed order)
+//      in a fixed tree over the ranks (the paper's global sum of partial forces)
 //      and run the FP64 corrector, Aarseth step and quantisation of the full path
 //      (same bits given the same forces); the smallest key of its chunk after the
 //      step is pushed into every CTA;
@@ -82,12 +83,12 @@ struct __align__(16) EngSmem {
     int2 qmap[kEngMaxS];                    // block position -> (owner rank, member index there)
     IRec own_rec[kEngCap];                  // this chunk's members' predicted records
     int own_idx[kEngCap];                   // this chunk's members (particle indices, ascending)
-    int rank_base[kEngMaxC];                // block position of each rank's first member
+    int own_hits;                           // number of them (may exceed kEngCap)
+    long long own_m2;                       // the chunk's smallest key other than the block time
     float2 red[kEngWarps][7];               // per-warp sums (blocks of up to 16)
     long long slot_min[kEngMaxC];           // written by rank q: the smallest key of its chunk after the step
     int slot_err[kEngMaxC];                 // written by rank q: its status bits of the step
     int slot_cnt[kEngMaxC];                 // written by rank q: its chunk's members of the block
-    int wcnt[kEngWarps];
     long long wmin[kEngWarps];
     int wflags[kEngWarps];
 };
@@ -106,14 +107,12 @@ __device__ __forceinline__ IPk ipk_of_rec(const IRec &R)
     return ipk_of(IPart{R.h.x, R.h.y, R.h.z, R.l.x, R.l.y, R.l.z, R.w.x, R.w.y, R.w.z});
 }
 
-// Sends the (hi, lo) partial sums of block position q to the member's owner.
-__device__ __forceinline__ void push_part(cg::cluster_group &cluster, EngSmem *sm, int q, int rank, const Acc7 &hi,
-                                          const Acc7 &lo)
+// Sends component c of the partial sums of block position q to the member's owner.
+__device__ __forceinline__ void push_part(cg::cluster_group &cluster, EngSmem *sm, int q, int rank, int c, float h,
+                                          float l)
 {
     const int2 o = sm->qmap[q];
-    float2 *dst = cluster.map_shared_rank(&sm->part_in[o.y][rank][0], o.x);
-#pragma unroll
-    for (int c = 0; c < 7; ++c) dst[c] = make_float2(acc_get(hi, c), acc_get(lo, c));
+    *cluster.map_shared_rank(&sm->part_in[o.y][rank][c], o.x) = make_float2(h, l);
 }
 
 // Partial sums of one member (predicted record ip, index gi) over pair records
@@ -160,8 +159,9 @@ __device__ void force_groups(cg::cluster_group &cluster, EngSmem *sm, const JPai
         zero(hi);
         zero(lo);
         sweep<true, TJ>(recs, j0, 0, nrec, tj, ip, gi, e2, hi, lo);
-        ds_group_reduce7<TJ>(hi, lo);
-        if (tj == 0 && q < s) push_part(cluster, sm, q, rank, hi, lo);
+        float h, l;
+        const int c = ds_scatter_reduce<TJ>(hi, lo, h, l);   // a lane ends with component c
+        if (c < 7 && q < s) push_part(cluster, sm, q, rank, c, h, l);
     }
 }
 
@@ -227,72 +227,80 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
         const DS tbs{tb2.x, tb2.y};
         if (!clean || steps >= budget || !(tb < kInfBits) || (E.check_end && !(tbd <= t_end))) break;
 
-        // ---- 1. this chunk's members (keys == block time), ascending, and the smallest other key
-        long long m2 = kInfBits;
-        int hits = 0;
-        for (int64_t c0 = j0; c0 < j1; c0 += 2 * kEngThreads) {
-            const int64_t e = c0 + 2 * (int64_t)tid;
-            const longlong2 kv = e < j1 ? *reinterpret_cast<const longlong2 *>(ckey + (e - j0))
-                                        : make_longlong2(kInfBits, kInfBits);
-            const bool h0 = kv.x == tb, h1 = kv.y == tb;
-            m2 = min_ll(m2, h0 ? kInfBits : kv.x);
-            m2 = min_ll(m2, h1 ? kInfBits : kv.y);
-            const unsigned b0 = __ballot_sync(full, h0), b1 = __ballot_sync(full, h1);
-            if (lane == 0) sm->wcnt[warp] = __popc(b0) + __popc(b1);
-            __syncthreads();
-            int woff = 0, tot = 0;
-#pragma unroll
-            for (int w = 0; w < kEngWarps; ++w) {
-                const int cw = sm->wcnt[w];
-                woff += w < warp ? cw : 0;
-                tot += cw;
+        // ---- 1., 2. Warp 0: the chunk's members (keys == block time), ascending, the smallest
+        // other key, the members' predicted records, pushed to every CTA. The other warps
+        // predict the whole chunk meanwhile (needed only if the block is taken, as it almost
+        // always is): neither waits for the other before the cluster barrier.
+        if (warp == 0) {
+            long long m2 = kInfBits;
+            int hits = 0;
+            for (int64_t c0 = j0; c0 < j1; c0 += 64) {
+                const int64_t e = c0 + 2 * (int64_t)lane;
+                const longlong2 kv = e < j1 ? *reinterpret_cast<const longlong2 *>(ckey + (e - j0))
+                                            : make_longlong2(kInfBits, kInfBits);
+                const bool h0 = kv.x == tb, h1 = kv.y == tb;
+                m2 = min_ll(m2, h0 ? kInfBits : kv.x);
+                m2 = min_ll(m2, h1 ? kInfBits : kv.y);
+                const unsigned b0 = __ballot_sync(full, h0), b1 = __ballot_sync(full, h1);
+                const unsigned below = (1u << lane) - 1u;
+                const int pos = hits + __popc(b0 & below) + __popc(b1 & below);
+                if (h0 && pos < kEngCap) sm->own_idx[pos] = (int)e;
+                if (h1 && pos + (h0 ? 1 : 0) < kEngCap) sm->own_idx[pos + (h0 ? 1 : 0)] = (int)(e + 1);
+                hits += __popc(b0) + __popc(b1);
             }
-            const unsigned below = (1u << lane) - 1u;
-            const int pos = hits + woff + __popc(b0 & below) + __popc(b1 & below);
-            if (h0 && pos < kEngCap) sm->own_idx[pos] = (int)e;
-            if (h1 && pos + (h0 ? 1 : 0) < kEngCap) sm->own_idx[pos + (h0 ? 1 : 0)] = (int)(e + 1);
-            hits += tot;
-            __syncthreads();   // wcnt is rewritten by the next segment
-        }
-        const int hk = hits < kEngCap ? hits : kEngCap;
-
-        // ---- 2. predict this chunk's members (the chunk itself only once the block is
-        // known to be taken) and push their records to every CTA
-        for (int q = tid; q < hk; q += kEngThreads) {
-            const int i = sm->own_idx[q];
-            const int64_t li = i - j0;
-            float2 X[3], V[3], Ac[3], K[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                X[c] = cx[c * ch + li];
-                V[c] = cv[c * ch + li];
-                Ac[c] = ca[c * ch + li];
-                K[c] = ck[c * ch + li];
+            m2 = warp_min(m2);
+            if (lane == 0) {
+                sm->own_hits = hits;
+                sm->own_m2 = m2;
             }
-            float4 h, l, w;
-            ds_predict_ds(X, V, Ac, K, ds_sub(tbs, DS{ct[li].x, ct[li].y}), h, l, w, cm[li]);
-            sm->own_rec[q] = IRec{make_float4(h.x, h.y, h.z, __int_as_float(i)), make_float4(l.x, l.y, l.z, 0.f),
-                                  make_float4(w.x, w.y, w.z, 0.f)};
+            __syncwarp();
+            const int hk = hits < kEngCap ? hits : kEngCap;
+            if (lane < hk) {
+                const int i = sm->own_idx[lane];
+                const int64_t li = i - j0;
+                float2 X[3], V[3], Ac[3], K[3];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    X[c] = cx[c * ch + li];
+                    V[c] = cv[c * ch + li];
+                    Ac[c] = ca[c * ch + li];
+                    K[c] = ck[c * ch + li];
+                }
+                float4 h, l, w;
+                ds_predict_ds(X, V, Ac, K, ds_sub(tbs, DS{ct[li].x, ct[li].y}), h, l, w, cm[li]);
+                sm->own_rec[lane] = IRec{make_float4(h.x, h.y, h.z, __int_as_float(i)),
+                                         make_float4(l.x, l.y, l.z, 0.f), make_float4(w.x, w.y, w.z, 0.f)};
+            }
+            __syncwarp();
+            if (!waited) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+            if (lane < C) *cluster.map_shared_rank(&sm->slot_cnt[rank], lane) = hits;
+            for (int q = lane; q < hk * C; q += 32) {
+                const int k = q / C, dst = q % C;
+                *cluster.map_shared_rank(&sm->inbox[rank][k], dst) = sm->own_rec[k];
+            }
+        } else {
+            if (!waited) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+            for (int64_t i = j0 + tid - 32; i < j1; i += kEngThreads - 32) {
+                const int64_t li = i - j0;
+                if (i < n) {
+                    float2 X[3], V[3], Ac[3], K[3];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        X[c] = cx[c * ch + li];
+                        V[c] = cv[c * ch + li];
+                        Ac[c] = ca[c * ch + li];
+                        K[c] = ck[c * ch + li];
+                    }
+                    float4 h, l, w;
+                    ds_predict_ds(X, V, Ac, K, ds_sub(tbs, DS{ct[li].x, ct[li].y}), h, l, w, cm[li]);
+                    jrec_store(recs, li, h.x, h.y, h.z, h.w, l.x, l.y, l.z, w.x, w.y, w.z);
+                } else {
+                    const float far = (float)kPadPos;
+                    jrec_store(recs, li, far, far, far, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
+                }
+            }
         }
-        // the corrector's FP64 state of this thread's member (four lanes per member),
-        // in flight during the force phase; a quad past the members works on member 0
-        // without storing (correct_group needs a valid particle, and one with the
-        // members' step keeps its fast path)
-        const int hq = tid >> 2;
-        const bool qlive = hq < hk;
-        const int icor = hk > 0 ? sm->own_idx[qlive ? hq : 0] : (int)j0;
-        GroupState gs{};
-        if (hk > 0 && warp * 8 < hk) gs = load_group(H, icor);
-        __syncthreads();
-        if (!waited) {
-            asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-            waited = true;
-        }
-        if (tid < C) *cluster.map_shared_rank(&sm->slot_cnt[rank], tid) = hits;
-        if (tid < hk * C) {
-            const int k = tid / C, dst = tid % C;
-            *cluster.map_shared_rank(&sm->inbox[rank][k], dst) = sm->own_rec[k];
-        }
+        waited = true;
         cluster.sync();
 
         // ---- the block: its size, this chunk's offset; does the engine take it?
@@ -310,42 +318,32 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
         }
         if (s < 1 || s > E.s_max || mx > kEngCap) break;
 
-        // ---- 3. the chunk's pair records; the members in block order (rank by rank);
-        // then the partial sums over this chunk, pushed to each member's owner
-        if (warp == 0) {
+        // ---- 3. the members in block order (rank by rank); then the partial sums over this
+        // chunk, pushed to each member's owner
+        const int hits = sm->own_hits;
+        const int hk = hits < kEngCap ? hits : kEngCap;
+        // the corrector's FP64 state of this thread's member (four lanes per member),
+        // in flight during the force phase; a quad past the members works on member 0
+        // without storing (correct_group needs a valid particle, and one with the
+        // members' step keeps its fast path)
+        const int hq = tid >> 2;
+        const bool qlive = hq < hk;
+        const int icor = hk > 0 ? sm->own_idx[qlive ? hq : 0] : (int)j0;
+        GroupState gs{};
+        if (hk > 0 && warp * 8 < hk) gs = load_group(H, icor);
+        {
+            // thread (r, k) places member k of rank r after the lower ranks' members
             const int cq = lane < C ? sm->slot_cnt[lane] : 0;
-            int incl = cq;
+            int before = cq;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(full, incl, o);
-                if (lane >= o) incl += y;
+                const int y = __shfl_up_sync(full, before, o);
+                if (lane >= o) before += y;
             }
-            if (lane < C) sm->rank_base[lane] = incl - cq;
-        }
-        for (int64_t i = j0 + tid; i < j1; i += kEngThreads) {
-            const int64_t li = i - j0;
-            if (i < n) {
-                float2 X[3], V[3], Ac[3], K[3];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    X[c] = cx[c * ch + li];
-                    V[c] = cv[c * ch + li];
-                    Ac[c] = ca[c * ch + li];
-                    K[c] = ck[c * ch + li];
-                }
-                float4 h, l, w;
-                ds_predict_ds(X, V, Ac, K, ds_sub(tbs, DS{ct[li].x, ct[li].y}), h, l, w, cm[li]);
-                jrec_store(recs, li, h.x, h.y, h.z, h.w, l.x, l.y, l.z, w.x, w.y, w.z);
-            } else {
-                const float far = (float)kPadPos;
-                jrec_store(recs, li, far, far, far, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
-            }
-        }
-        __syncthreads();
-        if (tid < C * kEngCap) {
-            const int r = tid / kEngCap, k = tid % kEngCap;
-            if (r < C && k < sm->slot_cnt[r]) {
-                const int q = sm->rank_base[r] + k;
+            before -= cq;
+            const int r = tid / kEngCap, k = tid % kEngCap;   // r < 32
+            const int q = __shfl_sync(full, before, r) + k, cnt = __shfl_sync(full, cq, r);
+            if (r < C && k < cnt) {
                 sm->ilist[q] = sm->inbox[r][k];
                 sm->qmap[q] = make_int2(r, k);
             }
@@ -366,16 +364,19 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
                 zero(hi);
                 zero(lo);
                 sweep<true, 32>(recs, j0, rb, re, lane, ip, gi, e2, hi, lo);
-                ds_group_reduce7<32>(hi, lo);
-                if (lane == 0) {
-#pragma unroll
-                    for (int c = 0; c < 7; ++c) sm->red[warp][c] = make_float2(acc_get(hi, c), acc_get(lo, c));
+                float h, l;
+                const int c = ds_scatter_reduce<32>(hi, lo, h, l);
+                if ((lane & 3) == 0 && c < 7) {
+                    if (G == 1)
+                        push_part(cluster, sm, q, rank, c, h, l);
+                    else
+                        sm->red[warp][c] = make_float2(h, l);
                 }
             }
-            __syncthreads();
+            if (G > 1) __syncthreads();   // (G is the same in every thread)
             // warp c adds component c of each member's G warp sums by a butterfly over
             // groups of G lanes (lane l holds warp l's sum; lanes past the members add zeros)
-            if (warp < 7) {
+            if (G > 1 && warp < 7) {
                 const int c = warp;
                 const bool has = lane < kEngWarps && lane / G < s;
                 float h = has ? sm->red[lane][c].x : 0.f, l = has ? sm->red[lane][c].y : 0.f;
@@ -383,10 +384,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
                     const float h2 = __shfl_xor_sync(full, h, off), l2 = __shfl_xor_sync(full, l, off);
                     ds_add(h, l, h2, l2);
                 }
-                if (has && lane % G == 0) {
-                    const int2 o = sm->qmap[lane / G];
-                    *cluster.map_shared_rank(&sm->part_in[o.y][rank][c], o.x) = make_float2(h, l);
-                }
+                if (has && lane % G == 0) push_part(cluster, sm, lane / G, rank, c, h, l);
             }
         } else {
             force_groups<8>(cluster, sm, recs, j0, j1, nrec, s, e2, rank);
@@ -396,7 +394,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
         // ---- 4. correct this chunk's members: the ranks' partial sums in rank order,
         // then the FP64 corrector
         int flags = 0;
-        long long tmin = m2;
+        long long tmin = kInfBits;
         if (warp * 8 < hk) {   // warps holding at least one member (quads 8w .. 8w + 7)
             const int c = (tid & 3) < 3 ? (tid & 3) : 2;
             const int k = qlive ? hq : 0;
@@ -406,15 +404,16 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
                 va[r] = r < C ? sm->part_in[k][r][c] : make_float2(0.f, 0.f);
                 vk[r] = r < C ? sm->part_in[k][r][3 + c] : make_float2(0.f, 0.f);
             }
-            float ha = 0.f, la = 0.f, hk_ = 0.f, lk = 0.f;
+            // a tree over the ranks (four dependent additions instead of sixteen)
 #pragma unroll
-            for (int r = 0; r < kEngMaxC; ++r) {
-                if (r < C) {
-                    ds_add(ha, la, va[r].x, va[r].y);
-                    ds_add(hk_, lk, vk[r].x, vk[r].y);
+            for (int d = 1; d < kEngMaxC; d <<= 1) {
+#pragma unroll
+                for (int r = 0; r < kEngMaxC; r += 2 * d) {
+                    ds_add(va[r].x, va[r].y, va[r + d].x, va[r + d].y);
+                    ds_add(vk[r].x, vk[r].y, vk[r + d].x, vk[r + d].y);
                 }
             }
-            const double an = (double)ha + (double)la, kn = (double)hk_ + (double)lk;
+            const double an = (double)va[0].x + (double)va[0].y, kn = (double)vk[0].x + (double)vk[0].y;
             long long newkey = kInfBits;
             flags |= correct_group(H, icor, gs, qlive, tbd, an, kn, A.eta, A.dt_max, A.dt_min, &newkey, &mir);
             tmin = min_ll(tmin, newkey);
@@ -442,7 +441,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
         // cluster reads them before the next kernel; this CTA's own next reads of
         // them follow a CTA barrier).
         if (warp == kEngWarps - 1) {
-            long long mm = lane < kEngWarps ? sm->wmin[lane] : kInfBits;
+            long long mm = lane < kEngWarps ? sm->wmin[lane] : sm->own_m2;
             int ff = lane < kEngWarps ? sm->wflags[lane] : 0;
             mm = warp_min(mm);
             ff = (int)__reduce_or_sync(full, (unsigned)ff);
