@@ -65,7 +65,7 @@ constexpr int kEngThreads = 512;
 constexpr int kEngWarps = kEngThreads / 32;
 constexpr int kEngMaxC = 16;
 constexpr long long kInfBits = 0x7ff0000000000000LL;
-static_assert(kEngCap <= 8 * (kEngWarps - 1), "the last warp must hold no member (four lanes per member)");
+static_assert(kEngCap == 16 && kEngWarps > 8, "two warps of members for each part of the correction, the last warp free");
 static_assert(kEngMaxC * kEngCap <= kEngThreads, "one thread per (rank, member) when pushing records");
 
 // predicted record of an active particle: (x_hi, y_hi, z_hi, index bits), (x_lo, y_lo, z_lo, 0), (vx, vy, vz, 0)
@@ -322,15 +322,17 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
         // chunk, pushed to each member's owner
         const int hits = sm->own_hits;
         const int hk = hits < kEngCap ? hits : kEngCap;
-        // the corrector's FP64 state of this thread's member (four lanes per member),
-        // in flight during the force phase; a quad past the members works on member 0
-        // without storing (correct_group needs a valid particle, and one with the
-        // members' step keeps its fast path)
-        const int hq = tid >> 2;
+        // the corrector's FP64 state of this thread's member (four lanes per member, and a
+        // pair of warps for each part of the correction), in flight during the force phase;
+        // a quad past the members works on member 0 without storing (the corrector needs a
+        // valid particle, and one with the members' step keeps its fast path)
+        const int part = warp >> 1;
+        const bool corrects = part < 4 && (warp & 1) * 8 < hk;   // this warp holds a member
+        const int hq = (tid & 63) >> 2;
         const bool qlive = hq < hk;
         const int icor = hk > 0 ? sm->own_idx[qlive ? hq : 0] : (int)j0;
         GroupState gs{};
-        if (hk > 0 && warp * 8 < hk) gs = load_group(H, icor);
+        if (corrects) gs = load_group(H, icor);
         {
             // thread (r, k) places member k of rank r after the lower ranks' members
             const int cq = lane < C ? sm->slot_cnt[lane] : 0;
@@ -392,10 +394,10 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
         cluster.sync();
 
         // ---- 4. correct this chunk's members: the ranks' partial sums in rank order,
-        // then the FP64 corrector
+        // then the FP64 corrector, its parts side by side
         int flags = 0;
         long long tmin = kInfBits;
-        if (warp * 8 < hk) {   // warps holding at least one member (quads 8w .. 8w + 7)
+        if (corrects) {
             const int c = (tid & 3) < 3 ? (tid & 3) : 2;
             const int k = qlive ? hq : 0;
             float2 va[kEngMaxC], vk[kEngMaxC];
@@ -415,7 +417,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
             }
             const double an = (double)va[0].x + (double)va[0].y, kn = (double)vk[0].x + (double)vk[0].y;
             long long newkey = kInfBits;
-            flags |= correct_group(H, icor, gs, qlive, tbd, an, kn, A.eta, A.dt_max, A.dt_min, &newkey, &mir);
+            flags |= correct_part(part, H, icor, gs, qlive, tbd, an, kn, A.eta, A.dt_max, A.dt_min, &newkey, &mir);
             tmin = min_ll(tmin, newkey);
         }
         tmin = warp_min(tmin);
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
             *A.interactions += (double)s * (double)n;
         }
         ++steps;
-        // The last warp (which holds no member: kEngCap members take warps 0 and 1)
+        // The last warp (which holds no member: the corrections take warps 0 to 7)
         // publishes this chunk's smallest key and status bits to every CTA and
         // arrives with release semantics; the other warps arrive relaxed, so the
         // barrier does not wait for the corrector's global stores (nothing in this

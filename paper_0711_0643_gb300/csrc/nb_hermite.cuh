@@ -172,7 +172,15 @@ __device__ __forceinline__ GroupState load_group(const HState &H, int64_t i)
     return GroupState{H.t[i], H.dt[i], H.x[o], H.v[o], H.a[o], H.k[o]};
 }
 
-__device__ __forceinline__ int correct_group(const HState &H, int64_t i, const GroupState &g, bool live, double tn,
+// The parts of a correction: the new step, time and key; the new position; the new
+// velocity; the new a and k. One particle's correction is a chain of some 1200
+// dependent instructions on one quad of lanes, latency-bound while few particles are
+// active; as parts on different warps (sub-partitions) the chain is a third as long,
+// at the price of forming a2 and a3 three times. Every value is the same, bit for bit.
+enum : int { kPartKey = 1, kPartX = 2, kPartV = 4, kPartAK = 8, kPartAll = 15 };
+
+template <int PARTS>
+__device__ __forceinline__ int correct_parts(const HState &H, int64_t i, const GroupState &g, bool live, double tn,
                                              double an, double kn, double eta, double dt_max, double dt_min,
                                              long long *key_out = nullptr, const DsMirror *mir = nullptr)
 {
@@ -194,22 +202,29 @@ __device__ __forceinline__ int correct_group(const HState &H, int64_t i, const G
     const double da = __dsub_rn(ao, an);
     const long long dtb = dbits(dt);
     const int e = (int)((dtb >> 52) & 0x7ff) - 1023;
-    double x1, v1, a2, a3;
-    if (__all_sync(full, dbits(d) == dtb && e >= -204 && e <= 204)) {
+    double x1 = 0.0, v1 = 0.0, a2 = 0.0, a3 = 0.0;
+    if (PARTS == kPartAK) {
+        // (no derivatives needed)
+    } else if (__all_sync(full, dbits(d) == dtb && e >= -204 && e <= 204)) {
         // d = dt = 2^e and every dt^k, 1/dt^k is a normal power of two: each product
         // with one of them (and with 2, 4, 1/2) is an exponent shift (scale2), the
         // same bits as the FP64 multiply below
         const double d2 = pow2_of(2 * e), d3 = pow2_of(3 * e), d4 = pow2_of(4 * e), d5 = pow2_of(5 * e);
         const double i1 = pow2_of(-e), i2 = pow2_of(-2 * e), i3 = pow2_of(-3 * e);
-        const double xp = __dadd_rn(__dadd_rn(__dadd_rn(x, scale2(v, e, dt)), scale2(scale2(ao, 2 * e, d2), -1, 0.5)),
-                                    rn_div6(scale2(ko, 3 * e, d3)));
-        const double vp = __dadd_rn(__dadd_rn(v, scale2(ao, e, dt)), scale2(scale2(ko, 2 * e, d2), -1, 0.5));
         // -6 da, 12 da and 6 (k_old + k_new) as exact integer products (same bits)
         a2 = __dsub_rn(scale2(dneg(rn_mul3(da, 1, 6.0)), -2 * e, i2),
                        scale2(__dadd_rn(scale2(ko, 2, 4.0), scale2(kn, 1, 2.0)), -e, i1));
         a3 = __dadd_rn(scale2(rn_mul3(da, 2, 12.0), -3 * e, i3), scale2(rn_mul3(__dadd_rn(ko, kn), 1, 6.0), -2 * e, i2));
-        x1 = __dadd_rn(__dadd_rn(xp, rn_div24(scale2(a2, 4 * e, d4))), rn_div120(scale2(a3, 5 * e, d5)));
-        v1 = __dadd_rn(__dadd_rn(vp, rn_div6(scale2(a2, 3 * e, d3))), rn_div24(scale2(a3, 4 * e, d4)));
+        if (PARTS & kPartX) {
+            const double xp = __dadd_rn(
+                __dadd_rn(__dadd_rn(x, scale2(v, e, dt)), scale2(scale2(ao, 2 * e, d2), -1, 0.5)),
+                rn_div6(scale2(ko, 3 * e, d3)));
+            x1 = __dadd_rn(__dadd_rn(xp, rn_div24(scale2(a2, 4 * e, d4))), rn_div120(scale2(a3, 5 * e, d5)));
+        }
+        if (PARTS & kPartV) {
+            const double vp = __dadd_rn(__dadd_rn(v, scale2(ao, e, dt)), scale2(scale2(ko, 2 * e, d2), -1, 0.5));
+            v1 = __dadd_rn(__dadd_rn(vp, rn_div6(scale2(a2, 3 * e, d3))), rn_div24(scale2(a3, 4 * e, d4)));
+        }
     } else {
         const double d2 = __dmul_rn(d, d);
         const double d3 = __dmul_rn(d2, d);
@@ -229,87 +244,105 @@ __device__ __forceinline__ int correct_group(const HState &H, int64_t i, const G
         x1 = __dadd_rn(__dadd_rn(xp, rn_div24(__dmul_rn(a2, dt4))), rn_div120(__dmul_rn(a3, dt5)));
         v1 = __dadd_rn(__dadd_rn(vp, rn_div6(__dmul_rn(a2, dt3))), rn_div24(__dmul_rn(a3, dt4)));
     }
-    const double a2p = __dadd_rn(a2, scale2(a3, e, dt));
-
-    // The step's power of two from the FP32 estimate. Lane q gathers the three
-    // component squares of vector q (a, k, a2p, a3) by rotating shuffles and sums
-    // them in component order, as dot3 does, in FP32 from RN32 copies of the FP64
-    // components made on the integer pipe (the estimate's error stays far inside
-    // its 2^-14 decision window). The FP64 norms are formed only where the
-    // estimate does not decide.
-    float c0f, c1f, c2f, c3f;
-    const bool ok32 = rn32_int(an, c0f) & rn32_int(kn, c1f) & rn32_int(a2p, c2f) & rn32_int(a3, c3f);
-    const float t0 = sq_ftz(c0f), t1 = sq_ftz(c1f), t2 = sq_ftz(c2f), t3 = sq_ftz(c3f);
-    float f0 = 0.f, f1 = 0.f, f2 = 0.f;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int w = (q - r) & 3;   // lane src supplies vector (src - r) & 3
-        const float mine = w == 0 ? t0 : (w == 1 ? t1 : (w == 2 ? t2 : t3));
-        const int src = (q + r) & 3;
-        const float got = __shfl_sync(full, mine, g0 + src);
-        if (src == 0) f0 = got;
-        if (src == 1) f1 = got;
-        if (src == 2) f2 = got;
-    }
-    const float fS = (f0 + f1) + f2;
-    const float rS = __fsqrt_rn(fS);
-    const float rA = __shfl_sync(full, rS, g0), rK = __shfl_sync(full, rS, g0 + 1);
-    const float rP = __shfl_sync(full, rS, g0 + 2), rQ = __shfl_sync(full, rS, g0 + 3);
-    const float fK = __shfl_sync(full, fS, g0 + 1), fP = __shfl_sync(full, fS, g0 + 2);
-    const unsigned okb = __ballot_sync(full, ok32 && norm2_f32_in_range(fS));
     long long qb = 0;
     bool pos = true;
-    bool decided = aarseth_estimate(rA, rK, rP, rQ, fK, fP, __double2float_rn(eta), qb);
-    decided = decided && ((okb >> g0) & 0xFu) == 0xFu;
-    if (__any_sync(full, live && !decided)) {
-        const double s0 = __dmul_rn(an, an), s1 = __dmul_rn(kn, kn), s2 = __dmul_rn(a2p, a2p),
-                     s3 = __dmul_rn(a3, a3);
-        double p0 = 0.0, p1 = 0.0, p2 = 0.0;
+    if (PARTS & kPartKey) {
+        const double a2p = __dadd_rn(a2, scale2(a3, e, dt));
+
+        // The step's power of two from the FP32 estimate. Lane q gathers the three
+        // component squares of vector q (a, k, a2p, a3) by rotating shuffles and sums
+        // them in component order, as dot3 does, in FP32 from RN32 copies of the FP64
+        // components made on the integer pipe (the estimate's error stays far inside
+        // its 2^-14 decision window). The FP64 norms are formed only where the
+        // estimate does not decide.
+        float c0f, c1f, c2f, c3f;
+        const bool ok32 = rn32_int(an, c0f) & rn32_int(kn, c1f) & rn32_int(a2p, c2f) & rn32_int(a3, c3f);
+        const float t0 = sq_ftz(c0f), t1 = sq_ftz(c1f), t2 = sq_ftz(c2f), t3 = sq_ftz(c3f);
+        float f0 = 0.f, f1 = 0.f, f2 = 0.f;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const double mine = pick4(s0, s1, s2, s3, (q - r) & 3);
+            const int w = (q - r) & 3;   // lane src supplies vector (src - r) & 3
+            const float mine = w == 0 ? t0 : (w == 1 ? t1 : (w == 2 ? t2 : t3));
             const int src = (q + r) & 3;
-            const double got = __shfl_sync(full, mine, g0 + src);
-            if (src == 0) p0 = got;
-            if (src == 1) p1 = got;
-            if (src == 2) p2 = got;
+            const float got = __shfl_sync(full, mine, g0 + src);
+            if (src == 0) f0 = got;
+            if (src == 1) f1 = got;
+            if (src == 2) f2 = got;
         }
-        const double S = __dadd_rn(__dadd_rn(p0, p1), p2);
-        const double mag = __dsqrt_rn(S);   // the four magnitudes, one per lane
-        const double mA = __shfl_sync(full, mag, g0), mK = __shfl_sync(full, mag, g0 + 1);
-        const double mP = __shfl_sync(full, mag, g0 + 2), mQ = __shfl_sync(full, mag, g0 + 3);
-        const double K = __shfl_sync(full, S, g0 + 1), P = __shfl_sync(full, S, g0 + 2);
-        if (!decided) {
-            const double num = __dadd_rn(__dmul_rn(mA, mP), K);
-            const double den = __dadd_rn(__dmul_rn(mK, mQ), P);
-            const double cand = den == 0.0 ? CUDART_INF : __dsqrt_rn(__ddiv_rn(__dmul_rn(eta, num), den));
-            qb = pow2_floor_bits(cand);
-            pos = dpositive(cand);
+        const float fS = (f0 + f1) + f2;
+        const float rS = __fsqrt_rn(fS);
+        const float rA = __shfl_sync(full, rS, g0), rK = __shfl_sync(full, rS, g0 + 1);
+        const float rP = __shfl_sync(full, rS, g0 + 2), rQ = __shfl_sync(full, rS, g0 + 3);
+        const float fK = __shfl_sync(full, fS, g0 + 1), fP = __shfl_sync(full, fS, g0 + 2);
+        const unsigned okb = __ballot_sync(full, ok32 && norm2_f32_in_range(fS));
+        bool decided = aarseth_estimate(rA, rK, rP, rQ, fK, fP, __double2float_rn(eta), qb);
+        decided = decided && ((okb >> g0) & 0xFu) == 0xFu;
+        if (__any_sync(full, live && !decided)) {
+            const double s0 = __dmul_rn(an, an), s1 = __dmul_rn(kn, kn), s2 = __dmul_rn(a2p, a2p),
+                         s3 = __dmul_rn(a3, a3);
+            double p0 = 0.0, p1 = 0.0, p2 = 0.0;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const double mine = pick4(s0, s1, s2, s3, (q - r) & 3);
+                const int src = (q + r) & 3;
+                const double got = __shfl_sync(full, mine, g0 + src);
+                if (src == 0) p0 = got;
+                if (src == 1) p1 = got;
+                if (src == 2) p2 = got;
+            }
+            const double S = __dadd_rn(__dadd_rn(p0, p1), p2);
+            const double mag = __dsqrt_rn(S);   // the four magnitudes, one per lane
+            const double mA = __shfl_sync(full, mag, g0), mK = __shfl_sync(full, mag, g0 + 1);
+            const double mP = __shfl_sync(full, mag, g0 + 2), mQ = __shfl_sync(full, mag, g0 + 3);
+            const double K = __shfl_sync(full, S, g0 + 1), P = __shfl_sync(full, S, g0 + 2);
+            if (!decided) {
+                const double num = __dadd_rn(__dmul_rn(mA, mP), K);
+                const double den = __dadd_rn(__dmul_rn(mK, mQ), P);
+                const double cand = den == 0.0 ? CUDART_INF : __dsqrt_rn(__ddiv_rn(__dmul_rn(eta, num), den));
+                qb = pow2_floor_bits(cand);
+                pos = dpositive(cand);
+            }
         }
     }
     int flags = 0;
     if (live) {
         if (q < 3) {
-            if (!(dfinite(x1) && dfinite(v1) && dfinite(an) && dfinite(kn))) flags |= kStNonfinite;
-            H.x[o] = x1;
-            H.v[o] = v1;
-            H.a[o] = an;
-            H.k[o] = kn;
+            if (PARTS & kPartX) {
+                if (!dfinite(x1)) flags |= kStNonfinite;
+                H.x[o] = x1;
+            }
+            if (PARTS & kPartV) {
+                if (!dfinite(v1)) flags |= kStNonfinite;
+                H.v[o] = v1;
+            }
+            if (PARTS & kPartAK) {
+                if (!(dfinite(an) && dfinite(kn))) flags |= kStNonfinite;
+                H.a[o] = an;
+                H.k[o] = kn;
+            }
             if (H.x2) {
-                const float2 px = rn_ds_pack(x1), pv = rn_ds_pack(v1), pa = rn_ds_pack(an), pk = rn_ds_pack(kn);
-                H.x2[o] = px;
-                H.v2[o] = pv;
-                H.a2[o] = pa;
-                H.k2[o] = pk;
-                if (mir) {
-                    const int64_t om = c * mir->np + (i - mir->base);
-                    mir->x2[om] = px;
-                    mir->v2[om] = pv;
-                    mir->a2[om] = pa;
-                    mir->k2[om] = pk;
+                const int64_t om = mir ? c * mir->np + (i - mir->base) : 0;
+                if (PARTS & kPartX) {
+                    const float2 px = rn_ds_pack(x1);
+                    H.x2[o] = px;
+                    if (mir) mir->x2[om] = px;
+                }
+                if (PARTS & kPartV) {
+                    const float2 pv = rn_ds_pack(v1);
+                    H.v2[o] = pv;
+                    if (mir) mir->v2[om] = pv;
+                }
+                if (PARTS & kPartAK) {
+                    const float2 pa = rn_ds_pack(an), pk = rn_ds_pack(kn);
+                    H.a2[o] = pa;
+                    H.k2[o] = pk;
+                    if (mir) {
+                        mir->a2[om] = pa;
+                        mir->k2[om] = pk;
+                    }
                 }
             }
-        } else {
+        } else if (PARTS & kPartKey) {
             const double dt_new = quantise_bits(qb, pos, dt, tn, dt_max, dt_min);
             if (dt_new == 0.0) flags |= kStUnderflow;
             const double key = __dadd_rn(tn, dt_new);
@@ -324,6 +357,24 @@ __device__ __forceinline__ int correct_group(const HState &H, int64_t i, const G
         }
     }
     return flags;
+}
+__device__ __forceinline__ int correct_group(const HState &H, int64_t i, const GroupState &g, bool live, double tn,
+                                             double an, double kn, double eta, double dt_max, double dt_min,
+                                             long long *key_out = nullptr, const DsMirror *mir = nullptr)
+{
+    return correct_parts<kPartAll>(H, i, g, live, tn, an, kn, eta, dt_max, dt_min, key_out, mir);
+}
+// Part `part` (0: key, 1: x, 2: v, 3: a and k; the same in all lanes of a warp).
+__device__ __forceinline__ int correct_part(int part, const HState &H, int64_t i, const GroupState &g, bool live,
+                                            double tn, double an, double kn, double eta, double dt_max, double dt_min,
+                                            long long *key_out = nullptr, const DsMirror *mir = nullptr)
+{
+    switch (part) {
+    case 0: return correct_parts<kPartKey>(H, i, g, live, tn, an, kn, eta, dt_max, dt_min, key_out, mir);
+    case 1: return correct_parts<kPartX>(H, i, g, live, tn, an, kn, eta, dt_max, dt_min, key_out, mir);
+    case 2: return correct_parts<kPartV>(H, i, g, live, tn, an, kn, eta, dt_max, dt_min, key_out, mir);
+    default: return correct_parts<kPartAK>(H, i, g, live, tn, an, kn, eta, dt_max, dt_min, key_out, mir);
+    }
 }
 __device__ __forceinline__ int correct_group(const HState &H, int64_t i, bool live, double tn, double an, double kn,
                                              double eta, double dt_max, double dt_min, long long *key_out = nullptr)

@@ -459,9 +459,14 @@ __device__ __forceinline__ void load_fin(const double *fin, int64_t ii, double *
     if (phi) *phi = p[6];
 }
 
-// Four lanes per active particle (correct_group): 32 particles per CTA and round.
+// Four lanes per active particle. Small blocks (one round of eight particles per CTA
+// covers them): every warp of a CTA does one part of the correction of the CTA's eight
+// particles (see correct_parts), the corrector being a chain of dependent instructions
+// then. Larger blocks: 32 particles per CTA and round, a quad doing all parts (fewer
+// FP64 instructions in all).
 constexpr int kCorThreads = 128;
 constexpr int kCorPer = kCorThreads / 4;
+constexpr int kCorSmall = 8;
 
 __global__ void __launch_bounds__(kCorThreads) correct_kernel(StepArgs A, int check_due, int lower_form)
 {
@@ -470,34 +475,46 @@ __global__ void __launch_bounds__(kCorThreads) correct_kernel(StepArgs A, int ch
     const HState H{A.x, A.v, A.a, A.k, A.t, A.dt, A.tn, A.x2, A.v2, A.a2, A.k2, A.n_pad};
     const int q = threadIdx.x & 3;
     const int c = q < 3 ? q : 2;
+    const bool small = s <= (int64_t)kCorSmall * gridDim.x;
+    const int per = small ? kCorSmall : kCorPer;
+    const int mine = small ? (threadIdx.x & 31) >> 2 : threadIdx.x >> 2;   // this quad's particle of a round
     // Launched programmatically after the force kernel (nb_run loop), this part
     // overlaps its end: the active list, the block time and the state were
     // written before it, only the new forces (fin) after. The first round's
     // particle and its state are read here; then wait for the force grid.
-    const int64_t base0 = (int64_t)blockIdx.x * kCorPer;
+    const int64_t base0 = (int64_t)blockIdx.x * per;
     int64_t i0 = 0;
     GroupState g0{};
     if (base0 < s) {
-        const int64_t ii = base0 + (threadIdx.x >> 2);
-        i0 = A.idx[ii < s ? ii : 0];
+        const int64_t ii = base0 + mine;
+        i0 = A.idx[ii < s ? ii : base0];
         g0 = load_group(H, i0);
+        if (small) __syncthreads();   // every part has read the state before one writes it
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");   // returns at once without such a dependency
     int flags = 0;
     long long kmin = 0x7ff0000000000000LL;   // smallest new key of this thread's particles
-    for (int64_t base = base0; base < s; base += (int64_t)gridDim.x * kCorPer) {
-        const int64_t ii = base + (threadIdx.x >> 2);
+    for (int64_t base = base0; base < s; base += (int64_t)gridDim.x * per) {
+        const int64_t ii = base + mine;
         bool live = ii < s;
-        const int64_t iis = live ? ii : 0;
+        const int64_t iis = live ? ii : base;
         const bool first = base == base0;
         const int64_t i = first ? i0 : A.idx[iis];
-        if (live && check_due && dbits(A.tn[i]) != dbits(tn)) {
-            live = false;
-            flags |= kStState;
+        if (check_due) {
+            const bool due = dbits(A.tn[i]) == dbits(tn);
+            if (small) __syncthreads();   // (and the key)
+            if (live && !due) {
+                live = false;
+                flags |= kStState;
+            }
         }
         const double an = A.fin[iis * kPartStride + c], kn = A.fin[iis * kPartStride + 3 + c];
         long long key = 0x7ff0000000000000LL;
-        flags |= correct_group(H, i, first ? g0 : load_group(H, i), live, tn, an, kn, A.eta, A.dt_max, A.dt_min, &key);
+        if (small)
+            flags |= correct_part(threadIdx.x >> 5, H, i, g0, live, tn, an, kn, A.eta, A.dt_max, A.dt_min, &key);
+        else
+            flags |= correct_group(H, i, first ? g0 : load_group(H, i), live, tn, an, kn, A.eta, A.dt_max, A.dt_min,
+                                   &key);
         kmin = key < kmin ? key : kmin;
     }
     if (lower_form) {
@@ -1023,9 +1040,10 @@ cudaError_t launch_select(const StepArgs &a, SelMode mode, unsigned long long co
 
 cudaError_t launch_correct(const StepArgs &a, bool check_due, bool lower_form, bool after_force, cudaStream_t st)
 {
-    // one round covers blocks of up to 608 * 32 particles; CTAs past s exit at once
+    // one round covers blocks of up to 608 * 32 particles (of up to 608 * 8 in parts); CTAs
+    // past s exit at once
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid_for(a.n, kCorPer, 608));
+    cfg.gridDim = dim3((unsigned)grid_for(a.n, kCorSmall, 608));
     cfg.blockDim = dim3(kCorThreads);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
