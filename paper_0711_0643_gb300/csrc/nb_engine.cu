@@ -126,6 +126,22 @@ __device__ __forceinline__ void sweep(const JPair *recs, int64_t j0, int rb, int
 {
     AccPk p;
     zero(p);
+    if (re - rb <= TJ * (kFoldPairs / 2)) {
+        // at most one fold's records per lane (chunks of up to 512 particles with TJ = 8):
+        // folding into empty accumulators is a copy
+#pragma unroll 4
+        for (int r = rb + tj; r < re; r += TJ) {
+            const float4 *Q = recs[r].q;
+            const int64_t ja = j0 + 2 * (int64_t)r;
+            pair_packed<MASK>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, MASK && ja == gi, MASK && ja + 1 == gi);
+        }
+        hi = Acc7{p.ax.x + p.ax.y, p.ay.x + p.ay.y, p.az.x + p.az.y, p.kx.x + p.kx.y,
+                  p.ky.x + p.ky.y, p.kz.x + p.kz.y, p.ph.x + p.ph.y};
+        zero(lo);
+        return;
+    }
+    zero(hi);
+    zero(lo);
     int cnt = 0;
 #pragma unroll 4
     for (int r = rb + tj; r < re; r += TJ) {
@@ -156,8 +172,6 @@ __device__ void force_groups(cg::cluster_group &cluster, EngSmem *sm, const JPai
         const int gi = __float_as_int(R.h.w);
         const IPk ip = ipk_of_rec(R);
         Acc7 hi, lo;
-        zero(hi);
-        zero(lo);
         sweep<true, TJ>(recs, j0, 0, nrec, tj, ip, gi, e2, hi, lo);
         float h, l;
         const int c = ds_scatter_reduce<TJ>(hi, lo, h, l);   // a lane ends with component c
@@ -363,8 +377,6 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
                 const IPk ip = ipk_of_rec(R);
                 const int rb = (int)((int64_t)nrec * part / G), re = (int)((int64_t)nrec * (part + 1) / G);
                 Acc7 hi, lo;
-                zero(hi);
-                zero(lo);
                 sweep<true, 32>(recs, j0, rb, re, lane, ip, gi, e2, hi, lo);
                 float h, l;
                 const int c = ds_scatter_reduce<32>(hi, lo, h, l);

@@ -19,7 +19,7 @@
 // corrects and scans the keys of its own chunk. Force work per block step: every
 // CTA takes all s active particles against its own chunk as j (the j-split,
 // j-share resident in shared memory for chunks of up to 1984 particles), and the
-// partials are summed in rank order by the CTA that owns each active particle;
+// partials are summed in a fixed tree by the CTA that owns each active particle;
 // blocks too large for the j-split's partial slots or shared-memory list (s >
 // kEnsSplitCap) are dealt out by i instead, each CTA taking a share of them
 // against all of the system's j (no reduction needed).
@@ -54,6 +54,8 @@ namespace {
 #endif
 constexpr int kEnsThreads = NB_ENS_THREADS;   // threads per CTA (and particles per j-tile)
 constexpr int kEnsTile = kEnsThreads;
+constexpr int kEnsPartMax = 16;               // members of a CTA corrected in parts (two warps a part)
+static_assert(kEnsThreads == 256, "eight warps: two for each part of a correction");
 // Largest block (active count s) taken by the j-split: every CTA runs all active
 // particles against its own j-share and the partials are summed across the
 // cluster, which needs C * s partial slots per cluster (8 float2 each) and the
@@ -337,6 +339,7 @@ __device__ __forceinline__ void share_pass(const EnsArgs &E, int64_t base, const
     zero(hi);
     zero(lo);
     const int nrec = ((nj + 1) / 2 + TJ - 1) / TJ;   // records per thread
+    const bool one = nrec <= FP;                     // folding into empty accumulators is a copy
     const int64_t self = (int64_t)gi - c0;           // i's place in the share, if it is there
     if (__any_sync(0xffffffffu, self >= 0 && self < nj)) {
         for (int k0 = 0; k0 < nrec; k0 += FP) {
@@ -347,7 +350,7 @@ __device__ __forceinline__ void share_pass(const EnsArgs &E, int64_t base, const
                 const float4 *Q = jb[pp].q;
                 pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, 2 * pp == self, 2 * pp + 1 == self);
             }
-            fold(hi, lo, p);
+            if (!one) fold(hi, lo, p);
         }
     } else {
         for (int k0 = 0; k0 < nrec; k0 += FP) {
@@ -357,14 +360,22 @@ __device__ __forceinline__ void share_pass(const EnsArgs &E, int64_t base, const
                 const float4 *Q = jb[tj + k * TJ].q;
                 pair_packed<false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, false, false);
             }
-            fold(hi, lo, p);
+            if (!one) fold(hi, lo, p);
         }
     }
-    if (TJ > 1) ds_group_reduce7<TJ>(hi, lo);
-    if (tj == 0 && live) {
-        float2 *dst = part + (slot0 + p0 + ti) * kPartStride;
+    if (one)
+        hi = Acc7{p.ax.x + p.ax.y, p.ay.x + p.ay.y, p.az.x + p.az.y, p.kx.x + p.kx.y,
+                  p.ky.x + p.ky.y, p.kz.x + p.kz.y, p.ph.x + p.ph.y};
+    // the group's sums; every lane ends with max(1, 8 / TJ) of the components
+    constexpr int N = TJ >= 8 ? 1 : 8 / TJ;
+    constexpr int kRun = TJ > 8 ? TJ / 8 : 1;   // lanes left with the same sum
+    float sh[N], sl[N];
+    const int first = ds_scatter_reduce<TJ, N>(hi, lo, sh, sl);
+    if (live && (tj & (kRun - 1)) == 0) {
+        float2 *dst = part + (slot0 + p0 + ti) * kPartStride + first;
 #pragma unroll
-        for (int c = 0; c < 7; ++c) dst[c] = make_float2(acc_get(hi, c), acc_get(lo, c));
+        for (int c = 0; c < N; ++c)
+            if (first + c < 7) dst[c] = make_float2(sh[c], sl[c]);
     }
 }
 
@@ -401,32 +412,38 @@ __device__ __noinline__ void share_force(const EnsArgs &E, int64_t base, const i
     }
 }
 
-// Component cq of a and k of list position p: the C ranks' partials summed in
-// rank order, all loads issued before the first addition.
+// Component cq of a and k of list position p: the C ranks' partials summed in a fixed
+// tree over the ranks, all loads issued before the first addition.
+template <int C>
+__device__ __forceinline__ void sum_partials_c(const float2 *part, int64_t s, int64_t p, int cq, double &an, double &kn)
+{
+    float2 va[C], vk[C];
+#pragma unroll
+    for (int u = 0; u < C; ++u) {
+        const float2 *src = part + ((int64_t)u * s + p) * kPartStride;
+        va[u] = __ldcg(src + cq);
+        vk[u] = __ldcg(src + 3 + cq);
+    }
+#pragma unroll
+    for (int d = 1; d < C; d <<= 1) {
+#pragma unroll
+        for (int u = 0; u < C; u += 2 * d) {
+            ds_add(va[u].x, va[u].y, va[u + d].x, va[u + d].y);
+            ds_add(vk[u].x, vk[u].y, vk[u + d].x, vk[u + d].y);
+        }
+    }
+    an = (double)va[0].x + (double)va[0].y;
+    kn = (double)vk[0].x + (double)vk[0].y;
+}
 __device__ __forceinline__ void sum_partials(const float2 *part, int64_t s, int64_t p, int cq, int C, double &an,
                                              double &kn)
 {
-    float ha = 0.f, la = 0.f, hk = 0.f, lk = 0.f;
-    for (int q0 = 0; q0 < C; q0 += 8) {
-        float2 va[8], vk[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (q0 + u < C) {
-                const float2 *src = part + ((int64_t)(q0 + u) * s + p) * kPartStride;
-                va[u] = __ldcg(src + cq);
-                vk[u] = __ldcg(src + 3 + cq);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (q0 + u < C) {
-                ds_add(ha, la, va[u].x, va[u].y);
-                ds_add(hk, lk, vk[u].x, vk[u].y);
-            }
-        }
+    switch (C) {   // the launch's cluster size
+    case 2: sum_partials_c<2>(part, s, p, cq, an, kn); break;
+    case 4: sum_partials_c<4>(part, s, p, cq, an, kn); break;
+    case 8: sum_partials_c<8>(part, s, p, cq, an, kn); break;
+    default: sum_partials_c<16>(part, s, p, cq, an, kn); break;
     }
-    an = (double)ha + (double)la;
-    kn = (double)hk + (double)lk;
 }
 
 // ---------------------------------------------------------------- phases
@@ -753,18 +770,35 @@ __global__ void __launch_bounds__(kEnsThreads, NB_ENS_MIN_BLOCKS) ensemble_kerne
                 cluster.sync();
                 if (tid == 0) sm->err = 0;
                 // each CTA corrects its own active particles (positions my_off ...
-                // my_off + my_cnt of the list), summing the ranks' partials in rank order
+                // my_off + my_cnt of the list), summing the ranks' partials in a fixed tree
                 const HState H{E.x, E.v, E.a, E.k, E.t, E.dt, E.tn, E.x2, E.v2, E.a2, E.k2, E.np};
-                for (int b0 = 0; b0 < my_cnt; b0 += kEnsThreads / 4) {
-                    const int kk = b0 + (tid >> 2);
-                    const bool live = kk < my_cnt;
-                    const int p = my_off + (live ? kk : 0);
-                    const int64_t i = base + slist[p];
-                    const GroupState g = load_group(H, i);
-                    double an, kn;
-                    sum_partials(part, s, p, cq, C, an, kn);
-                    flags |= correct_group(H, i, g, live, tblock, an, kn, E.eta, E.dt_max, E.dt_min);
-                    if (live && (tid & 3) == 3) E.t2[i] = rn_ds_pack(tblock);
+                if (my_cnt <= kEnsPartMax) {
+                    // few: the parts of a correction on different warps (correct_parts),
+                    // a pair of warps for each; all have read the state before one writes
+                    if (my_cnt > 0) {
+                        const int kk = (tid & 63) >> 2;
+                        const bool live = kk < my_cnt;
+                        const int p = my_off + (live ? kk : 0);
+                        const int64_t i = base + slist[p];
+                        const GroupState g = load_group(H, i);
+                        double an, kn;
+                        sum_partials(part, s, p, cq, C, an, kn);
+                        __syncthreads();
+                        flags |= correct_part(warp >> 1, H, i, g, live, tblock, an, kn, E.eta, E.dt_max, E.dt_min);
+                        if (tid < 64 && live && (tid & 3) == 3) E.t2[i] = rn_ds_pack(tblock);
+                    }
+                } else {
+                    for (int b0 = 0; b0 < my_cnt; b0 += kEnsThreads / 4) {
+                        const int kk = b0 + (tid >> 2);
+                        const bool live = kk < my_cnt;
+                        const int p = my_off + (live ? kk : 0);
+                        const int64_t i = base + slist[p];
+                        const GroupState g = load_group(H, i);
+                        double an, kn;
+                        sum_partials(part, s, p, cq, C, an, kn);
+                        flags |= correct_group(H, i, g, live, tblock, an, kn, E.eta, E.dt_max, E.dt_min);
+                        if (live && (tid & 3) == 3) E.t2[i] = rn_ds_pack(tblock);
+                    }
                 }
                 // the keys and states just written belong to this CTA: a CTA barrier
                 // orders them before the next scan and prediction
