@@ -117,9 +117,8 @@ __device__ __forceinline__ void push_part(cg::cluster_group &cluster, EngSmem *s
 
 // Partial sums of one member (predicted record ip, index gi) over pair records
 // [rb, re) of the chunk, lanes interleaved with stride TJ starting at lane tj.
-// MASK: the member's own pair is left out by index (the engine always masks: one
-// instantiation per width keeps the kernel's code, and its instruction-cache
-// footprint, small).
+// MASK: the member's own pair is left out by index (only where it would not be an exact
+// zero, see self_is_zero). The potential is not formed: the corrector needs a and k.
 template <bool MASK, int TJ>
 __device__ __forceinline__ void sweep(const JPair *recs, int64_t j0, int rb, int re, int tj, const IPk &ip, int gi,
                                       float2 e2, Acc7 &hi, Acc7 &lo)
@@ -133,10 +132,10 @@ __device__ __forceinline__ void sweep(const JPair *recs, int64_t j0, int rb, int
         for (int r = rb + tj; r < re; r += TJ) {
             const float4 *Q = recs[r].q;
             const int64_t ja = j0 + 2 * (int64_t)r;
-            pair_packed<MASK>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, MASK && ja == gi, MASK && ja + 1 == gi);
+            pair_packed<MASK, false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, MASK && ja == gi, MASK && ja + 1 == gi);
         }
         hi = Acc7{p.ax.x + p.ax.y, p.ay.x + p.ay.y, p.az.x + p.az.y, p.kx.x + p.kx.y,
-                  p.ky.x + p.ky.y, p.kz.x + p.kz.y, p.ph.x + p.ph.y};
+                  p.ky.x + p.ky.y, p.kz.x + p.kz.y, 0.f};
         zero(lo);
         return;
     }
@@ -148,7 +147,7 @@ __device__ __forceinline__ void sweep(const JPair *recs, int64_t j0, int rb, int
         const float4 *Q = recs[r].q;
         const float4 q0 = Q[0], q1 = Q[1], q2 = Q[2], q3 = Q[3], q4 = Q[4];
         const int64_t ja = j0 + 2 * (int64_t)r;
-        pair_packed<MASK>(q0, q1, q2, q3, q4, ip, e2, p, MASK && ja == gi, MASK && ja + 1 == gi);
+        pair_packed<MASK, false>(q0, q1, q2, q3, q4, ip, e2, p, MASK && ja == gi, MASK && ja + 1 == gi);
         if (++cnt == kFoldPairs / 2) {
             cnt = 0;
             fold(hi, lo, p);
@@ -161,7 +160,7 @@ __device__ __forceinline__ void sweep(const JPair *recs, int64_t j0, int rb, int
 // takes members in rounds; the group's lanes reduce with two-sums in a fixed order.
 template <int TJ>
 __device__ void force_groups(cg::cluster_group &cluster, EngSmem *sm, const JPair *recs, int64_t j0, int64_t j1,
-                             int nrec, int s, float2 e2, int rank)
+                             const float *cm, int nrec, int s, float2 e2, int rank)
 {
     constexpr int kGroups = kEngThreads / TJ;
     const int tid = threadIdx.x, tj = tid % TJ, g = tid / TJ;
@@ -172,10 +171,13 @@ __device__ void force_groups(cg::cluster_group &cluster, EngSmem *sm, const JPai
         const int gi = __float_as_int(R.h.w);
         const IPk ip = ipk_of_rec(R);
         Acc7 hi, lo;
-        sweep<true, TJ>(recs, j0, 0, nrec, tj, ip, gi, e2, hi, lo);
+        if (__any_sync(0xffffffffu, gi >= j0 && gi < j1 && !self_is_zero(e2.x, cm[gi - j0])))
+            sweep<true, TJ>(recs, j0, 0, nrec, tj, ip, gi, e2, hi, lo);
+        else
+            sweep<false, TJ>(recs, j0, 0, nrec, tj, ip, gi, e2, hi, lo);
         float h, l;
         const int c = ds_scatter_reduce<TJ>(hi, lo, h, l);   // a lane ends with component c
-        if (c < 7 && q < s) push_part(cluster, sm, q, rank, c, h, l);
+        if (c < 6 && q < s) push_part(cluster, sm, q, rank, c, h, l);
     }
 }
 
@@ -377,10 +379,13 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
                 const IPk ip = ipk_of_rec(R);
                 const int rb = (int)((int64_t)nrec * part / G), re = (int)((int64_t)nrec * (part + 1) / G);
                 Acc7 hi, lo;
-                sweep<true, 32>(recs, j0, rb, re, lane, ip, gi, e2, hi, lo);
+                if (gi >= j0 && gi < j1 && !self_is_zero(e2.x, cm[gi - j0]))   // (the same in the warp)
+                    sweep<true, 32>(recs, j0, rb, re, lane, ip, gi, e2, hi, lo);
+                else
+                    sweep<false, 32>(recs, j0, rb, re, lane, ip, gi, e2, hi, lo);
                 float h, l;
                 const int c = ds_scatter_reduce<32>(hi, lo, h, l);
-                if ((lane & 3) == 0 && c < 7) {
+                if ((lane & 3) == 0 && c < 6) {
                     if (G == 1)
                         push_part(cluster, sm, q, rank, c, h, l);
                     else
@@ -390,7 +395,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
             if (G > 1) __syncthreads();   // (G is the same in every thread)
             // warp c adds component c of each member's G warp sums by a butterfly over
             // groups of G lanes (lane l holds warp l's sum; lanes past the members add zeros)
-            if (G > 1 && warp < 7) {
+            if (G > 1 && warp < 6) {
                 const int c = warp;
                 const bool has = lane < kEngWarps && lane / G < s;
                 float h = has ? sm->red[lane][c].x : 0.f, l = has ? sm->red[lane][c].y : 0.f;
@@ -401,7 +406,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) engine_kernel(EngineArgs E)
                 if (has && lane % G == 0) push_part(cluster, sm, lane / G, rank, c, h, l);
             }
         } else {
-            force_groups<8>(cluster, sm, recs, j0, j1, nrec, s, e2, rank);
+            force_groups<8>(cluster, sm, recs, j0, j1, cm, nrec, s, e2, rank);
         }
         cluster.sync();
 

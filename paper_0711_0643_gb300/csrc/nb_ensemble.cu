@@ -341,14 +341,15 @@ __device__ __forceinline__ void share_pass(const EnsArgs &E, int64_t base, const
     const int nrec = ((nj + 1) / 2 + TJ - 1) / TJ;   // records per thread
     const bool one = nrec <= FP;                     // folding into empty accumulators is a copy
     const int64_t self = (int64_t)gi - c0;           // i's place in the share, if it is there
-    if (__any_sync(0xffffffffu, self >= 0 && self < nj)) {
+    // (the potential is not formed: the corrector needs a and k only)
+    if (__any_sync(0xffffffffu, self >= 0 && self < nj && !self_is_zero(eps2f, h.w))) {
         for (int k0 = 0; k0 < nrec; k0 += FP) {
             const int k1 = k0 + FP < nrec ? k0 + FP : nrec;
 #pragma unroll 4
             for (int k = k0; k < k1; ++k) {
                 const int pp = tj + k * TJ;
                 const float4 *Q = jb[pp].q;
-                pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, 2 * pp == self, 2 * pp + 1 == self);
+                pair_packed<true, false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, 2 * pp == self, 2 * pp + 1 == self);
             }
             if (!one) fold(hi, lo, p);
         }
@@ -358,14 +359,14 @@ __device__ __forceinline__ void share_pass(const EnsArgs &E, int64_t base, const
 #pragma unroll 4
             for (int k = k0; k < k1; ++k) {
                 const float4 *Q = jb[tj + k * TJ].q;
-                pair_packed<false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, false, false);
+                pair_packed<false, false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, false, false);
             }
             if (!one) fold(hi, lo, p);
         }
     }
     if (one)
         hi = Acc7{p.ax.x + p.ax.y, p.ay.x + p.ay.y, p.az.x + p.az.y, p.kx.x + p.kx.y,
-                  p.ky.x + p.ky.y, p.kz.x + p.kz.y, p.ph.x + p.ph.y};
+                  p.ky.x + p.ky.y, p.kz.x + p.kz.y, 0.f};
     // the group's sums; every lane ends with max(1, 8 / TJ) of the components
     constexpr int N = TJ >= 8 ? 1 : 8 / TJ;
     constexpr int kRun = TJ > 8 ? TJ / 8 : 1;   // lanes left with the same sum
@@ -375,7 +376,7 @@ __device__ __forceinline__ void share_pass(const EnsArgs &E, int64_t base, const
         float2 *dst = part + (slot0 + p0 + ti) * kPartStride + first;
 #pragma unroll
         for (int c = 0; c < N; ++c)
-            if (first + c < 7) dst[c] = make_float2(sh[c], sl[c]);
+            if (first + c < 6) dst[c] = make_float2(sh[c], sl[c]);
     }
 }
 

@@ -977,26 +977,37 @@ __device__ __forceinline__ void share_pass(const ForceArgs &A, Smem *sm, int64_t
     zero(p);
     zero(hi);
     zero(lo);
-    // i's place in the share, if it is there (else a value no record matches);
-    // one loop with the self test in it keeps the code small: each launch runs
-    // its passes once, from a cold instruction cache
-    const int64_t self = (int64_t)gi - 2 * rec0;
-    const int selfi = self >= 0 && self < 2 * (int64_t)nrec ? (int)self : -2;
+    // the round holding i's own record, if this thread meets it
+    const int64_t self = ((int64_t)gi >> 1) - rec0;
+    const int selfk = self >= 0 && self < (int64_t)nrec && (int)self % TJ == tj ? (int)self / TJ : -1;
     const JPair *R = shb(sm)->rec;
     for (int k0 = 0; k0 < nr; k0 += FP) {
         const int k1 = k0 + FP < nr ? k0 + FP : nr;
+        if (__any_sync(0xffffffffu, selfk >= k0 && selfk < k1)) {
 #pragma unroll 2
-        for (int k = k0; k < k1; ++k) {
-            const int pp = tj + k * TJ;
-            const float4 *Q = R[pp].q;
-            pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, 2 * pp == selfi, 2 * pp + 1 == selfi);
+            for (int k = k0; k < k1; ++k) {
+                const float4 *Q = R[tj + k * TJ].q;
+                pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, k == selfk && !(gi & 1),
+                                  k == selfk && (gi & 1));
+            }
+        } else {
+#pragma unroll 2
+            for (int k = k0; k < k1; ++k) {
+                const float4 *Q = R[tj + k * TJ].q;
+                pair_packed<false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, false, false);
+            }
         }
         fold(hi, lo, p);
     }
-    if (TJ > 1) ds_group_reduce7<TJ>(hi, lo);
-    if (tj == 0 && live) {
+    // the group's sums; every lane ends with max(1, 8 / TJ) of the components
+    constexpr int N = TJ >= 8 ? 1 : 8 / TJ;
+    constexpr int kRun = TJ > 8 ? TJ / 8 : 1;   // lanes left with the same sum
+    float sh[N], sl[N];
+    const int first = ds_scatter_reduce<TJ, N>(hi, lo, sh, sl);
+    if (live && (tj & (kRun - 1)) == 0) {
 #pragma unroll
-        for (int c = 0; c < 7; ++c) shb(sm)->slot[slot0 + ti][c] = make_float2(acc_get(hi, c), acc_get(lo, c));
+        for (int c = 0; c < N; ++c)
+            if (first + c < 7) shb(sm)->slot[slot0 + ti][first + c] = make_float2(sh[c], sl[c]);
     }
 }
 
@@ -1036,11 +1047,7 @@ __device__ __forceinline__ void share_pass_wide(const ForceArgs &A, Smem *sm, in
         }
     }
     fold(hi, lo, p);
-    ds_group_reduce7<32>(hi, lo);
-    if (lane == 0) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) sm->red[warp][c] = make_float2(acc_get(hi, c), acc_get(lo, c));
-    }
+    cta_sum_red(hi, lo, sm->red[warp]);
     __syncthreads();
     if (tid < cnt * 7) {
         const int t = tid / 7, c = tid % 7;

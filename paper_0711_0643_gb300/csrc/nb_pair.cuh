@@ -268,8 +268,9 @@ __device__ __forceinline__ void zero(AccPk &q)
     q.ax = q.ay = q.az = q.kx = q.ky = q.kz = q.ph = z;
 }
 
-// MASK zeroes lane a (j = 2p) or b (j = 2p+1) when it is the i-particle itself.
-template <bool MASK>
+// MASK zeroes lane a (j = 2p) or b (j = 2p+1) when it is the i-particle itself. PHI:
+// with the potential (the integration loops need none).
+template <bool MASK, bool PHI = true>
 __device__ __forceinline__ void pair_packed(const float4 &q0, const float4 &q1, const float4 &q2, const float4 &q3,
                                             const float4 &q4, const IPk &I, float2 eps2, AccPk &A, bool self_a,
                                             bool self_b)
@@ -294,13 +295,22 @@ __device__ __forceinline__ void pair_packed(const float4 &q0, const float4 &q1, 
     const float2 mq = __fmul2_rn(make_float2(q1.z, q1.w), q);
     const float2 mu = __fmul2_rn(mq, qq);
     const float2 nal = __fmul2_rn(__fmul2_rn(rw, make_float2(-3.f, -3.f)), qq);
-    A.ph = __ffma2_rn(mq, make_float2(-1.f, -1.f), A.ph);
+    if (PHI) A.ph = __ffma2_rn(mq, make_float2(-1.f, -1.f), A.ph);
     A.ax = __ffma2_rn(mu, dx, A.ax);
     A.ay = __ffma2_rn(mu, dy, A.ay);
     A.az = __ffma2_rn(mu, dz, A.az);
     A.kx = __ffma2_rn(mu, __ffma2_rn(nal, dx, wx), A.kx);
     A.ky = __ffma2_rn(mu, __ffma2_rn(nal, dy, wy), A.ky);
     A.kz = __ffma2_rn(mu, __ffma2_rn(nal, dz, wz), A.kz);
+}
+
+// Whether a particle of mass m need not be left out of its own sums of a and k: the
+// pair with its own record has r = w = 0 exactly, so its terms are exact zeros as long
+// as m (r^2 + eps^2)^(-3/2) is finite (the potential's term is not zero).
+__device__ __forceinline__ bool self_is_zero(float eps2, float m)
+{
+    const float q = rsqrtf(eps2);
+    return eps2 > 0.f && fabsf(m) * q * (q * q) < 1e36f;   // NaN and overflow: false
 }
 
 // both lanes of the packed partial into the (hi, lo) two-sum accumulator; p = 0 after
