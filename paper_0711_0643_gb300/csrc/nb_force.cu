@@ -100,13 +100,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int64_
 // ------------------------------------------------------------ shared memory
 
 constexpr int kPT = kJT / 2;    // pair records per tile
-constexpr int kRing = 6;        // tiles in flight in the TMA streaming variant
+constexpr int kRing = 8;        // tiles in flight in the TMA streaming variant
 
 // Column kernel (see there): a unit is up to kUnitRec pair records in kUnitBytes of
 // shared memory, kSlots units in flight.
 constexpr int kUnitRec = 256;
 constexpr int kUnitBytes = kUnitRec * (int)sizeof(JPair);
 constexpr int kSlots = 4;
+constexpr int kLongTiles = 12;  // variant 0: items of this many tiles go through the TMA ring (the same sums;
+                                // N = 2^20, s = 1, particles from HBM: 16.9 -> 16.5 us, no difference at 8)
 constexpr int kShortTiles = 32; // shares of up to this many tiles may go by whole items (see short_items)
 
 // Resident-share variant: clusters of kShareC CTAs, CTA r holding up to
@@ -244,6 +246,20 @@ __device__ __forceinline__ void copy_list(const ForceArgs &A, int64_t s)
     if (blockIdx.x == 0 && threadIdx.x == 0) *A.s_copy = s;
 }
 
+template <int U>
+__device__ __forceinline__ void sum_lane(const float2 *src, int lane, int n, float &h, float &l)
+{
+    for (int q0 = lane; q0 < n; q0 += 32 * U) {
+        float2 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            v[u] = q0 + 32 * u < n ? __ldcg(src + (q0 + 32 * u) * kPartStride) : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (q0 + 32 * u < n) ds_add(h, l, v[u].x, v[u].y);
+    }
+}
+
 // Adds the n partials of each of the active particles [ib0, ib1) (slots 0 .. n - 1 of S)
 // by this CTA, in a fixed order, and writes the results.
 __device__ void sum_parts(const ForceArgs &A, int64_t ib0, int64_t ib1, int S, int n)
@@ -251,21 +267,14 @@ __device__ void sum_parts(const ForceArgs &A, int64_t ib0, int64_t ib1, int S, i
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int np = (int)(ib1 - ib0);
     if (np == 1) {
-        // a warp per component; lane l adds partials l, l + 32, ... (kUnroll loads per
-        // round), then a butterfly of two-sums over the lanes
-        constexpr int kUnroll = 4;
+        // a warp per component; lane l adds partials l, l + 32, ..., their loads issued
+        // together (ten cover a partial from every CTA), then a butterfly over the lanes
         if (warp < 7) {
-            const float2 *src = part2(A, ib0, 0, S) + warp;
             float h = 0.f, l = 0.f;
-            for (int q0 = lane; q0 < n; q0 += 32 * kUnroll) {
-                float2 v[kUnroll];
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u)
-                    v[u] = q0 + 32 * u < n ? __ldcg(src + (q0 + 32 * u) * kPartStride) : make_float2(0.f, 0.f);
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u)
-                    if (q0 + 32 * u < n) ds_add(h, l, v[u].x, v[u].y);
-            }
+            if (n <= 64)
+                sum_lane<2>(part2(A, ib0, 0, S) + warp, lane, n, h, l);
+            else
+                sum_lane<10>(part2(A, ib0, 0, S) + warp, lane, n, h, l);
             ds_group_reduce<32>(h, l);
             if (lane == 0) put_final(A, ib0, warp, (double)h + (double)l);
         }
@@ -1252,7 +1261,7 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
             work_stream<2>(A, w, sm);
         else if (variant == 2)
             work_tile32(A, w, sm, git);
-        else if (variant == 0)
+        else if (variant == 0 && sm->tper < kLongTiles)
             work_stream<1>(A, w, sm);
         else
             work_stream_tma(A, w, sm, git);
