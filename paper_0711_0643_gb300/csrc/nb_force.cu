@@ -117,6 +117,8 @@ constexpr int kShortTiles = 32; // shares of up to this many tiles may go by who
 constexpr int kShareC = 8;
 constexpr int kShareRec = 1024;
 constexpr int kShareSlots = 256;
+constexpr int kSharePiece = 256;   // records per copy (four mbarriers)
+static_assert(kShareRec / kSharePiece <= kRing, "one mbarrier per piece");
 
 // How the column kernel cuts a launch (worked out by one thread per CTA).
 struct ColPlan {
@@ -159,7 +161,9 @@ struct __align__(128) Smem {
 
 struct ShareBuf {
     JPair rec[kShareRec];            // this CTA's share of the j-records
-    float2 slot[kShareSlots][7];     // (hi, lo) partials of the chunk's particles
+    // (hi, lo) partials of the chunk's positions rank, rank + kShareC, ..., pushed here by
+    // every CTA of the cluster
+    float2 in[kShareSlots / kShareC][kShareC][7];
 };
 
 constexpr size_t kSmemShare =
@@ -951,15 +955,18 @@ __host__ __device__ __forceinline__ int mixed_I(int v)
 // ------------------------------------------------- resident-share variant
 // For j ranges of up to kShareC * kShareRec pair records. The launch runs as
 // clusters of kShareC CTAs; CTA r of a cluster copies records [r * rper, (r + 1)
-// * rper) of the range into shared memory once (bulk copies on one mbarrier),
-// padded with far-away massless records to whole rounds of 32. The clusters deal
-// out the active list in chunks (chunk k to cluster k mod clusters); every CTA of
-// the cluster runs the whole chunk against its share in passes whose group
-// width TJ fits the remaining count, leaving (hi, lo) partials in its shared
-// memory. After a cluster barrier, CTA r sums positions r, r + kShareC, ... of
-// the chunk over the kShareC CTAs in rank order through distributed shared
-// memory and writes the FP64 results; a second barrier frees the slots. No
-// global partial slots, tickets or fences; the same bits on every run.
+// * rper) of the range into shared memory once (bulk copies of kSharePiece records, each
+// on its own mbarrier: the first pass starts on the first piece), padded with far-away
+// massless records to whole rounds of 32. The clusters deal out the active list in
+// chunks (chunk k to cluster k mod clusters); every CTA of the cluster runs the whole
+// chunk against its share in passes whose group width TJ fits the remaining count, and
+// pushes each position's (hi, lo) partial sums into the shared memory of the CTA that
+// finishes it (position mod kShareC). One cluster barrier later that CTA adds the
+// kShareC partials from its own shared memory, in a fixed tree over the ranks, and
+// writes the FP64 results. No global partial slots, tickets or fences; the same bits on
+// every run. Bound by latency up to a few hundred particles; us under the profiler, with
+// one wait for the whole share, partials read across the cluster after the barrier and a
+// second barrier / now: N = 16384, s = 20 9.2 / 7.9, 100 12.7 / 11.0, 256 14.6 / 14.0, 2000 55.2 / 54.0.
 
 // rper: records per CTA, a multiple of 32 (0 when the range does not fit)
 __device__ __forceinline__ int64_t share_rper(const ForceArgs &A)
@@ -969,13 +976,33 @@ __device__ __forceinline__ int64_t share_rper(const ForceArgs &A)
     return rper <= kShareRec ? rper : 0;
 }
 
-// One pass: cnt particles from list position p0 into slots slot0 ..., TJ threads
+// Waits for the share's pieces up to the one holding record r (ready: pieces this thread
+// has waited for). On a timeout the status is set and the copy gets a second wait, so that
+// none is in flight when the CTA ends.
+__device__ __forceinline__ void share_wait(const ForceArgs &A, Smem *sm, int r, int &ready)
+{
+    for (const int need = r / kSharePiece + 1; ready < need; ++ready)
+        if (!mbar_wait(&sm->bar[ready], 0, A.spin_limit)) {
+            atomicOr(A.status, kStTimeout);
+            (void)mbar_wait(&sm->bar[ready], 0, A.spin_limit);
+        }
+}
+
+// Sends component c of the partial sums of chunk position pl to the CTA that finishes it.
+__device__ __forceinline__ void share_push(Smem *sm, int rank, int pl, int c, float h, float l)
+{
+    cg::cluster_group cl = cg::this_cluster();
+    *cl.map_shared_rank(&shb(sm)->in[pl / kShareC][rank][c], pl % kShareC) = make_float2(h, l);
+}
+
+// One pass: cnt particles from list position p0, chunk positions slot0 ..., TJ threads
 // per particle taking records tj, tj + TJ, ... of the share (nr rounds).
 template <int TJ>
 __device__ __forceinline__ void share_pass(const ForceArgs &A, Smem *sm, int64_t p0, int cnt, int slot0,
-                                           int64_t rec0, int nrec, int nr)
+                                           int64_t rec0, int nrec, int nr, int rank, int &ready)
 {
-    constexpr int FP = kFoldPairs / 2;   // records per fold
+    constexpr int FP = kFoldPairs / 2;   // rounds per fold
+    constexpr int STEP = kSharePiece / TJ < FP ? kSharePiece / TJ : FP;   // rounds of one piece, within a fold
     const int tid = threadIdx.x, tj = tid % TJ, ti = tid / TJ;
     const bool live = ti < cnt;
     const int32_t gi = idx_at(A, sm, p0 + (live ? ti : cnt - 1));
@@ -990,8 +1017,11 @@ __device__ __forceinline__ void share_pass(const ForceArgs &A, Smem *sm, int64_t
     const int64_t self = ((int64_t)gi >> 1) - rec0;
     const int selfk = self >= 0 && self < (int64_t)nrec && (int)self % TJ == tj ? (int)self / TJ : -1;
     const JPair *R = shb(sm)->rec;
-    for (int k0 = 0; k0 < nr; k0 += FP) {
-        const int k1 = k0 + FP < nr ? k0 + FP : nr;
+    // the first pass follows the pieces as they arrive, the later ones go fold by fold
+    const int step = ready < kShareRec / kSharePiece ? STEP : FP;
+    for (int k0 = 0; k0 < nr; k0 += step) {
+        const int k1 = k0 + step < nr ? k0 + step : nr;
+        share_wait(A, sm, k1 * TJ - 1, ready);
         if (__any_sync(0xffffffffu, selfk >= k0 && selfk < k1)) {
 #pragma unroll 2
             for (int k = k0; k < k1; ++k) {
@@ -1006,7 +1036,7 @@ __device__ __forceinline__ void share_pass(const ForceArgs &A, Smem *sm, int64_t
                 pair_packed<false>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, false, false);
             }
         }
-        fold(hi, lo, p);
+        if (k1 % FP == 0 || k1 == nr) fold(hi, lo, p);
     }
     // the group's sums; every lane ends with max(1, 8 / TJ) of the components
     constexpr int N = TJ >= 8 ? 1 : 8 / TJ;
@@ -1016,19 +1046,21 @@ __device__ __forceinline__ void share_pass(const ForceArgs &A, Smem *sm, int64_t
     if (live && (tj & (kRun - 1)) == 0) {
 #pragma unroll
         for (int c = 0; c < N; ++c)
-            if (first + c < 7) shb(sm)->slot[slot0 + ti][first + c] = make_float2(sh[c], sl[c]);
+            if (first + c < 7) share_push(sm, rank, slot0 + ti, first + c, sh[c], sl[c]);
     }
 }
 
-// A pass for cnt <= 4 particles with 256 / cnt threads each (whole warps): lanes
-// then warps of a particle summed in ascending order.
+// A pass for cnt <= 8 / W particles with W warps each: lanes then warps of a particle
+// summed in ascending order. The rounds of one piece at a time, side by side.
+template <int W>
 __device__ __forceinline__ void share_pass_wide(const ForceArgs &A, Smem *sm, int64_t p0, int cnt, int slot0,
-                                                int64_t rec0, int nrec, int nrec32)
+                                                int64_t rec0, int nrec, int nrec32, int rank, int &ready)
 {
     constexpr int FP = kFoldPairs / 2;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int W = cnt == 1 ? 8 : (cnt == 2 ? 4 : 2);   // warps per particle
-    const int TW = 32 * W;                            // threads per particle
+    constexpr int TW = 32 * W;               // threads per particle
+    constexpr int G = kSharePiece / TW;      // rounds per piece
+    static_assert(kShareRec / TW <= FP, "one fold");
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int ti = tid / TW, tj = tid % TW;
     const bool live = ti < cnt;
     const int32_t gi = idx_at(A, sm, p0 + (live ? ti : cnt - 1));
@@ -1042,17 +1074,15 @@ __device__ __forceinline__ void share_pass_wide(const ForceArgs &A, Smem *sm, in
     const int64_t self = (int64_t)gi - 2 * rec0;
     const int selfi = self >= 0 && self < 2 * (int64_t)nrec ? (int)self : -2;
     const JPair *R = shb(sm)->rec;
-    const int nr = (nrec32 + TW - 1) / TW;
-    int f = 0;
-    for (int k = 0; k < nr; ++k) {
-        const int pp = tj + k * TW;
-        if (pp < nrec32) {
-            const float4 *Q = R[pp].q;
-            pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, 2 * pp == selfi, 2 * pp + 1 == selfi);
-        }
-        if (++f == FP) {
-            f = 0;
-            fold(hi, lo, p);
+    for (int b0 = 0; b0 < nrec32; b0 += kSharePiece) {
+        share_wait(A, sm, b0, ready);
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            const int pp = b0 + u * TW + tj;
+            if (pp < nrec32) {
+                const float4 *Q = R[pp].q;
+                pair_packed<true>(Q[0], Q[1], Q[2], Q[3], Q[4], ip, e2, p, 2 * pp == selfi, 2 * pp + 1 == selfi);
+            }
         }
     }
     fold(hi, lo, p);
@@ -1061,8 +1091,9 @@ __device__ __forceinline__ void share_pass_wide(const ForceArgs &A, Smem *sm, in
     if (tid < cnt * 7) {
         const int t = tid / 7, c = tid % 7;
         float h = sm->red[t * W][c].x, l = sm->red[t * W][c].y;
+#pragma unroll
         for (int wv = 1; wv < W; ++wv) ds_add(h, l, sm->red[t * W + wv][c].x, sm->red[t * W + wv][c].y);
-        shb(sm)->slot[slot0 + t][c] = make_float2(h, l);
+        share_push(sm, rank, slot0 + t, c, h, l);
     }
     __syncthreads();
 }
@@ -1080,85 +1111,84 @@ __device__ __noinline__ void share_force(const ForceArgs &A, int64_t s, Smem *sm
     const int nrec = (int)(rec0 < rlim ? (rlim - rec0 < rper ? rlim - rec0 : rper) : 0);
     const int nrec32 = (nrec + 31) / 32 * 32;
     // chunks: ceil(s / clusters) particles each (at most kShareSlots)
-    int64_t csz = (s + ncl - 1) / ncl;
+    int64_t csz = qdiv(s + ncl - 1, ncl);
     if (csz > kShareSlots) csz = kShareSlots;
-    const int64_t nchunk = (s + csz - 1) / csz;
+    const int64_t nchunk = qdiv(s + csz - 1, csz);
     if (q >= nchunk) return;   // the whole cluster has nothing to do (uniform over it)
-    // the share: bulk copies of at most 16 KB on one mbarrier, padding by the threads
-    bool ok = true;
-    if (nrec > 0) {
-        if (tid == 0) {
-            const uint32_t bytes = (uint32_t)nrec * (uint32_t)sizeof(JPair);
-            mbar_arrive_expect_tx(&sm->bar[0], bytes);
-            constexpr int kPiece = 200;   // records per copy (16000 bytes)
-            for (int r0 = 0; r0 < nrec; r0 += kPiece) {
-                const int nr = nrec - r0 < kPiece ? nrec - r0 : kPiece;
-                bulk_g2s(shb(sm)->rec + r0, A.j.p + rec0 + r0, (uint32_t)nr * (uint32_t)sizeof(JPair), &sm->bar[0]);
-            }
-        }
+    // no CTA writes into another's shared memory before all of the cluster run: arrive
+    // here, wait before the first pass
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    if (tid < kShareRec / kSharePiece) {
+        // (a piece past the share completes at once)
+        const int r0 = tid * kSharePiece;
+        const int nr = nrec - r0 < kSharePiece ? nrec - r0 : kSharePiece;
+        const uint32_t bytes = nr > 0 ? (uint32_t)nr * (uint32_t)sizeof(JPair) : 0u;
+        mbar_arrive_expect_tx(&sm->bar[tid], bytes);
+        if (nr > 0) bulk_g2s(shb(sm)->rec + r0, A.j.p + rec0 + r0, bytes, &sm->bar[tid]);
     }
     {
         const float far = (float)kPadPos;
         for (int qq = 2 * nrec + tid; qq < 2 * nrec32; qq += kThreads)
             jrec_store(shb(sm)->rec, qq, far, far, far, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
     }
-    if (nrec > 0 && !mbar_wait(&sm->bar[0], 0, A.spin_limit)) {
-        ok = false;
-        if (tid == 0) atomicOr(A.status, kStTimeout);
-    }
     __syncthreads();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    int ready = 0;
     for (int64_t k = q; k < nchunk; k += ncl) {
         const int64_t c0 = k * csz;
         const int cnt = (int)(c0 + csz < s ? csz : s - c0);
-        if (ok) {
-            int done = 0;
-            while (done < cnt) {
-                const int r = cnt - done;
-                if (r >= 256) {
-                    share_pass<1>(A, sm, c0 + done, 256, done, rec0, nrec, nrec32);
-                    done += 256;
-                } else if (r >= 128) {
-                    share_pass<2>(A, sm, c0 + done, 128, done, rec0, nrec, nrec32 / 2);
-                    done += 128;
-                } else if (r >= 64) {
-                    share_pass<4>(A, sm, c0 + done, 64, done, rec0, nrec, nrec32 / 4);
-                    done += 64;
-                } else if (r >= 32) {
-                    share_pass<8>(A, sm, c0 + done, 32, done, rec0, nrec, nrec32 / 8);
-                    done += 32;
-                } else if (r > 8) {
-                    const int n16 = r < 16 ? r : 16;
-                    share_pass<16>(A, sm, c0 + done, n16, done, rec0, nrec, nrec32 / 16);
-                    done += n16;
-                } else if (r > 4) {
-                    share_pass<32>(A, sm, c0 + done, r, done, rec0, nrec, nrec32 / 32);
-                    done += r;
-                } else {
-                    share_pass_wide(A, sm, c0 + done, r, done, rec0, nrec, nrec32);
-                    done += r;
-                }
+        int done = 0;
+        while (done < cnt) {
+            const int r = cnt - done;
+            if (r >= 256) {
+                share_pass<1>(A, sm, c0 + done, 256, done, rec0, nrec, nrec32, rank, ready);
+                done += 256;
+            } else if (r >= 128) {
+                share_pass<2>(A, sm, c0 + done, 128, done, rec0, nrec, nrec32 / 2, rank, ready);
+                done += 128;
+            } else if (r >= 64) {
+                share_pass<4>(A, sm, c0 + done, 64, done, rec0, nrec, nrec32 / 4, rank, ready);
+                done += 64;
+            } else if (r >= 32) {
+                share_pass<8>(A, sm, c0 + done, 32, done, rec0, nrec, nrec32 / 8, rank, ready);
+                done += 32;
+            } else if (r > 8) {
+                const int n16 = r < 16 ? r : 16;
+                share_pass<16>(A, sm, c0 + done, n16, done, rec0, nrec, nrec32 / 16, rank, ready);
+                done += n16;
+            } else if (r > 4) {
+                share_pass<32>(A, sm, c0 + done, r, done, rec0, nrec, nrec32 / 32, rank, ready);
+                done += r;
+            } else {
+                if (r == 1)
+                    share_pass_wide<8>(A, sm, c0 + done, r, done, rec0, nrec, nrec32, rank, ready);
+                else if (r == 2)
+                    share_pass_wide<4>(A, sm, c0 + done, r, done, rec0, nrec, nrec32, rank, ready);
+                else
+                    share_pass_wide<2>(A, sm, c0 + done, r, done, rec0, nrec, nrec32, rank, ready);
+                done += r;
             }
-        } else {
-            for (int qq = tid; qq < cnt * 7; qq += kThreads)
-                shb(sm)->slot[qq / 7][qq % 7] = make_float2(0.f, 0.f);
         }
-        cl.sync();
-        // rank r sums positions r, r + kShareC, ...: one (position, component) per thread
+        cl.sync();   // every CTA's partials are in the finishing CTAs' shared memory
+        // positions rank, rank + kShareC, ...: one (position, component) per thread
         for (int t = tid; t < ((cnt + kShareC - 1) / kShareC) * 7; t += kThreads) {
             const int pl = rank + kShareC * (t / 7), c = t % 7;
             if (pl < cnt) {
                 float2 v[kShareC];
 #pragma unroll
-                for (int u = 0; u < kShareC; ++u) v[u] = *cl.map_shared_rank(&shb(sm)->slot[pl][c], u);
-                float h = 0.f, l = 0.f;
+                for (int u = 0; u < kShareC; ++u) v[u] = shb(sm)->in[t / 7][u][c];
 #pragma unroll
-                for (int u = 0; u < kShareC; ++u) ds_add(h, l, v[u].x, v[u].y);
-                put_final(A, c0 + pl, c, (double)h + (double)l);
+                for (int d = 1; d < kShareC; d <<= 1) {
+#pragma unroll
+                    for (int u = 0; u < kShareC; u += 2 * d) ds_add(v[u].x, v[u].y, v[u + d].x, v[u + d].y);
+                }
+                put_final(A, c0 + pl, c, (double)v[0].x + (double)v[0].y);
             }
         }
-        cl.sync();
+        if (k + ncl < nchunk) cl.sync();   // the partials have been read: the next chunk may push
     }
-    if (!ok && nrec > 0 && tid == 0) (void)mbar_wait(&sm->bar[0], 0, A.spin_limit);   // drain before exit
+    // a CTA whose passes met no record of a piece still waits for its copy before it ends
+    share_wait(A, sm, kShareRec - 1, ready);
 }
 
 // Variants 1 and 2 where one item (two or eight particles, one share) per CTA covers the
