@@ -566,7 +566,7 @@ __device__ void work_stream_tma(const ForceArgs &A, int64_t w, Smem *sm, uint32_
 // alone would take 76), i.e. 8.9e11 pairs/s. Measured against items of (i-block, share)
 // with 1, 2, 8, 32 or 256 particles, dealt out in advance (us a call): N = 65536: s = 480
 // 71.3 -> 59.4, 1024 150 -> 100, 5000 862 -> 417, N 5850 -> 5010; N = 200000, s = 700 298
-// -> 196; N = 300007: s = 33 49 -> 31, 61 47.9 -> 40.9; N = 2^20: s = 64 115 -> 108, 1024
+// -> 196; N = 300007: s = 33 49 -> 31, 61 47.9 -> 39.6; N = 2^20: s = 64 115 -> 104, 1024
 // 1424 -> 1300; N = s = 131072 20480 -> 19990 (94 clocks a record).
 
 __device__ __forceinline__ int variant_lgst(int v) { return v == 1 ? 8 : (v == 2 ? 5 : (v == 3 ? 3 : 0)); }
@@ -775,9 +775,11 @@ __device__ bool work_cols(const ForceArgs &A, int64_t s, Smem *sm)
     const int ncol = lgnu ? 1 : 1 << (P.lgcw - lgtj);      // of them per unit
     const int c0 = tj & (cstep - 1);
     const int mine = lgnu ? tj >> P.lgcw : 0;              // this thread's unit of a round
-    // slots are refilled one round behind, when all warps have most likely left them
-    // (rounds of more than half of the slots: at once)
-    const int ahead = kSlots - ((2 << lgnu) <= kSlots ? 1 << lgnu : 0);
+    // Slots are refilled one unit behind, when all warps have most likely left it. Rounds of
+    // several units: at once (the warp whose turn it is waits for the slowest), so that the
+    // next round's units are on their way. One round behind they were not: N = 300007, s =
+    // 61 39.4 -> 37.5 us under the profiler, N = 2^20, s = 61 103 -> 100.6.
+    const int ahead = kSlots - (lgnu == 0 ? 1 : 0);
     const int hop = P.lgst == 0 ? (int)sizeof(JPair) : (int)sizeof(JPair) << P.lgcw;
     const int chop = P.lgst == 0 ? 32 * (int)sizeof(JPair) : (int)sizeof(JPair);
     const float2 e2 = make_float2(A.eps2f, A.eps2f);
