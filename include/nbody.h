@@ -265,7 +265,9 @@ nb_status nb_sync(nb_ctx *ctx);
  * bucket (bucket b holds s in (2^(b-1), 2^b]); variant -1 restores the default.
  * split is the j-split factor at the bucket's largest size min(2^b, n); a
  * smaller block of the bucket keeps the same number of work items (i-blocks x
- * splits), so its split grows in proportion.
+ * splits), so its split grows in proportion. It sets which FP32 partial sums are
+ * formed; mixed variants 1 to 4 and FP64 share the work out in equal runs over
+ * the GPU whatever it is.
  * nb_get_tuning reads the table (variant[32], split[32]). */
 nb_status nb_autotune(nb_ctx *ctx);
 nb_status nb_set_tuning(nb_ctx *ctx, int32_t bucket, int32_t variant, int32_t split);
