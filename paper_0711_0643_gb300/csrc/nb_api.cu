@@ -222,7 +222,9 @@ cudaError_t launch_force_ctx(nb_ctx *c)
 // steps (~16 us at N = 16384, mostly the FP64 corrector chain and the barrier-
 // separated phases on 16 SMs) plus a launch each time a large block interrupts
 // it cost as much as the four-kernel steps (Plummer N = 16384 to t = 1: 686 vs
-// 674 ms), while at N = 1024 it saves a fifth (58 vs 75 ms).
+// 674 ms), while at N = 1024 it saved a fifth (58 vs 75 ms). Both have become faster
+// since (N = 1024 to t = 1/4 13.2 -> 10.8 ms, N = 16384 to t = 1/16 39.0 -> 36 ms); the
+// line stays, as it also decides which FP32 partial sums a run forms.
 int32_t default_engine_smax(int64_t n)
 {
     if (n > kEngDefaultMaxN) return 0;
