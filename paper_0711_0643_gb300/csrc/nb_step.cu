@@ -664,7 +664,7 @@ __global__ void set_active_kernel(const int32_t *src, int32_t *dst, int64_t s, i
 // terms in double-single on the FP32 pipe (an FP64 instruction costs ~64 FP32 lanes'
 // worth here). Every pair once: i-block b (kEnThreads particles, one per thread)
 // takes the j's after its own first particle, in units of kEnUnit j's; the pairs with
-// j <= i of its first kEnThreads j's count as zero. All (i-block, unit) pairs are laid
+// j <= i of its first kEnThreads j's, and the half of an odd last record, count as zero. All (i-block, unit) pairs are laid
 // out in one line and cut into equal runs, one per CTA, so every SM has the same work
 // whatever n; FP64 takes over per particle (m_i phi_i), for the CTA's sums and for the
 // total, which the last CTA adds up in CTA order (fixed order: the same bits on
@@ -804,7 +804,9 @@ __global__ void __launch_bounds__(kEnThreads, 7) energy_kernel(StepArgs A, doubl
             __syncthreads();
             {
                 const int64_t j = jt + tid;
-                const bool real = j < j1;   // massless far-away records past the end add exact zeros
+                // an odd last record is filled up with anything: the masked loop below leaves it out
+                // (a massless far-away particle would not do: 0 / r is NaN where r^2 overflows)
+                const bool real = j < j1;
                 const float far = (float)kPadPos;
                 const float2 xj = real ? A.x2[j] : make_float2(far, 0.f), yj = real ? A.x2[np + j] : make_float2(far, 0.f),
                              zj = real ? A.x2[2 * np + j] : make_float2(far, 0.f);
@@ -823,10 +825,10 @@ __global__ void __launch_bounds__(kEnThreads, 7) energy_kernel(StepArgs A, doubl
             __syncthreads();
             const int64_t left = j1 - jt;
             const int np2 = (int)((left < kEnThreads ? left : kEnThreads) + 1) / 2;
-            if (jt < i0 + kEnThreads) {
+            if (jt < i0 + kEnThreads || left < kEnThreads) {
                 for (int q = 0; q < np2; ++q)
                     en_pair2<true>(sj[0][q], sj[1][q], sj[2][q], sj[3][q], I, e2h, e2l, jt + 2 * q > i,
-                                   jt + 2 * q + 1 > i, h, l);
+                                   jt + 2 * q + 1 > i && jt + 2 * q + 1 < j1, h, l);
             } else {
                 for (int q = 0; q < np2; ++q)
                     en_pair2<false>(sj[0][q], sj[1][q], sj[2][q], sj[3][q], I, e2h, e2l, true, true, h, l);
