@@ -813,10 +813,15 @@ __device__ bool work_cols(const ForceArgs &A, int64_t s, Smem *sm)
             // a round: 2^lgnu units (the last one of an i-block or run may have fewer)
             const int cnt = ue - u < (1 << lgnu) ? (int)(ue - u) : 1 << lgnu;
             const bool have = mine < cnt;
-            const uint32_t v = used + (uint32_t)(have ? mine : 0);
-            const int sl = (int)(v % kSlots);
-            ok = mbar_wait(&sm->bar[sl], (v / kSlots) & 1u, A.spin_limit);
+            // The warp releases all the units of the round, so it waits for all their copies, not
+            // only for its own unit's. Only then are the slots' earlier phases behind it: another
+            // warp's releases of one round come from different lanes and may be seen in any
+            // order, and a wait tests one parity bit, so that otherwise a release could count for
+            // the phase before, or the refill's wait below pass on the phase two before.
+            for (uint32_t v = used; v < used + (uint32_t)cnt; ++v)
+                ok = mbar_wait(&sm->bar[v % kSlots], (v / kSlots) & 1u, A.spin_limit) && ok;
             if (__all_sync(0xffffffffu, ok)) {
+                const int sl = (int)((used + (uint32_t)(have ? mine : 0)) % kSlots);
                 const int2 q = sm->info[sl];
                 const bool self = have && u + mine == su;
                 const unsigned char *src = sm->unit[sl] + c0 * chop;
