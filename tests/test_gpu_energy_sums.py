@@ -1,6 +1,9 @@
 """The energy's sums where their arithmetic could give out, against direct FP64 sums: odd
 particle counts far from the origin (the last record of two particles is half empty, and
-nothing in the other half may reach the sum)."""
+nothing in the other half may reach the sum), and rows of half a million terms that do not
+average out over the particles."""
+import math
+
 import numpy as np
 import pytest
 
@@ -36,3 +39,24 @@ def test_odd_count_far_from_the_origin(nb, orc, n):
     assert abs(K - Kr) <= 1e-14 * abs(Kr)
     assert abs(W - Wr) <= 1e-12 * abs(Wr)      # n = 1: both are 0
     assert E == K + W
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_one_heavy_body_holds_a_long_row(nb, seed):
+    """Body 0 holds all but 2^-51 of the mass, so W is its own row to 2^-51. Tolerance: a pair
+    term is within 2^-43, and the row's additions leave below 1e-13 (2^18 terms a lane, rms
+    in an FP32 emulation): 1e-12."""
+    n, eps = (1 << 19) + 3, 1.0 / 64
+    rng = ics.SplitMix64(900 + seed)
+    x = rng.uniform(3 * n).reshape(n, 3) * 2.0 - 1.0
+    v = rng.uniform(3 * n).reshape(n, 3) - 0.5
+    m = 2.0 ** -70 * (0.5 + rng.uniform(n))
+    m[0] = 1.0
+    r = np.sqrt(((x[1:] - x[0]) ** 2).sum(1) + eps * eps)
+    Wr = -math.fsum(m[1:] / r)
+    Kr = 0.5 * math.fsum(m * (v * v).sum(1))
+    with nb.Context() as c:
+        nb.nb_init(c.ctx, m, x, v, eps * eps)
+        E, K, W = nb.nb_energy(c.ctx)
+    assert abs(K - Kr) <= 1e-14 * Kr
+    assert abs(W - Wr) <= 1e-12 * abs(Wr), (W - Wr) / Wr
