@@ -26,6 +26,7 @@
 
 #include "nb_internal.cuh"
 #include "nb_pair.cuh"
+#include "nb_rsqrt.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -1330,23 +1331,6 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
 // with at most n_tiles / 4 shares of j above, so 16 of 152 SMs at work at N = 16384):
 // N = 16384: s = 1 18.4 -> 12.3, 64 84 -> 74, 256 2278 -> 250 (the pipe's time for its
 // instructions is 213), N 18020 -> 15310; N = 65536, s = 1024 4587 -> 3820.
-
-// (r2)^(-1/2) by a third-order Householder step from an FP32 estimate q0:
-// e = 1 - r2 q0^2 (q0^2 is exact in FP64 and the difference rounds once, |e| < 2^-21),
-// q = q0 + q0 e (1/2 + 3/8 e), truncation below 2^-64 relative, so q is the correctly
-// rounded value to within a few hundredths of an ulp. The conversions to and from
-// FP32 are moves of the bit fields (FP64 conversions share the narrow pipe). Only
-// where r2 is not comfortably a normal FP32 number: the library function.
-__device__ __forceinline__ double rsqrt_f64(double r2)
-{
-    const int hi = __double2hiint(r2);
-    if ((unsigned)(hi - ((1023 - 120) << 20)) >= (unsigned)(240 << 20)) return rsqrt(r2);
-    const float f = __int_as_float(__funnelshift_l(__double2loint(r2), hi - (896 << 20), 3));
-    const int qb = __float_as_int(rsqrtf(f));
-    const double q0 = __hiloint2double((qb >> 3) + (896 << 20), qb << 29);
-    const double e = fma(-r2, q0 * q0, 1.0);
-    return fma(q0 * e, fma(e, 0.375, 0.5), q0);
-}
 
 __device__ __forceinline__ void pair_f64(double xj, double yj, double zj, double mj, double vxj, double vyj,
                                          double vzj, const double *xi, double eps2, double *acc, bool self)
