@@ -48,13 +48,28 @@ __device__ __forceinline__ double d2_of(double ux, double uy, double uz, double 
 // operands of the packed instructions on two stars).
 struct __align__(16) Bin {
     float4 x, y, z;          // -cm as double-single: (hi, hi, lo, lo) per component
-    float4 k;                // (-K, -K, w K, w K): K = d^6 / (gamma m_b)^2
+    float4 k;                // (-K, -K, w K, w K): K = d^6 / (gamma m_b)^2 4^e
     double cm[3], d6, rhs;
     int i, j;                // members; i < 0: an invalid pair (or none)
     float K, cabs;           // K (0: invalid pair, NaN: the FP32 test never decides), |cm_x| + |cm_y| + |cm_z|
 };
 
-__device__ void load_bin(const PertArgs &P, int32_t b, Bin &q)
+// The masses are scaled by 2^-e for the FP32 test, K by 4^e: the same sides. e = 0 unless
+// the first and the last star are both outside the masses it takes (see star_tm2), which
+// then stand for the unit of mass: without it a call whose stars are all outside pays for
+// both tests (N = 16384, 1638 binaries, masses times 2^22: 877 us, 832 with the FP64 test
+// alone, now 61).
+constexpr int kMassLo = -34, kMassBits = 42;   // |m| 2^-e in [2^-34, 2^8)
+__device__ __forceinline__ int mass_exp(const PertArgs &P)
+{
+    if (P.j_lo >= P.j_hi) return 0;
+    const int a = ((__double2hiint(P.m[P.j_lo]) >> 20) & 0x7ff) - 1023;
+    const int z = ((__double2hiint(P.m[P.j_hi - 1]) >> 20) & 0x7ff) - 1023;
+    const bool fits = (unsigned)(a - kMassLo) < kMassBits || (unsigned)(z - kMassLo) < kMassBits;
+    return fits || z < -120 || z > 120 ? 0 : z;
+}
+
+__device__ void load_bin(const PertArgs &P, int32_t b, int e, Bin &q)
 {
     const float nan = __int_as_float(0x7fffffff);
     q.i = q.j = -1;
@@ -84,17 +99,18 @@ __device__ void load_bin(const PertArgs &P, int32_t b, Bin &q)
     q.d6 = __dmul_rn(__dmul_rn(d2, d2), d2);
     const double gm = __dmul_rn(P.gamma, mb);
     q.rhs = __dmul_rn(gm, gm);
-    // FP64 sides that could leave the normal range, and a K outside [2^-55, 2^100], are
-    // not for the FP32 test
-    const bool normal = q.d6 >= 0x1p-800 && q.d6 <= 0x1p800 && q.rhs >= 0x1p-800 && q.rhs <= 0x1p800;
-    const double K = __ddiv_rn(q.d6, q.rhs);
+    // FP64 sides that could leave the normal range (their masses are up to 2^128 where e is
+    // not 0), and a K outside [2^-55, 2^100], are not for the FP32 test
+    const double top = e == 0 ? 0x1p800 : 0x1p600, low = e == 0 ? 0x1p-800 : 0x1p-600;
+    const bool normal = q.d6 >= low && q.d6 <= top && q.rhs >= low && q.rhs <= top;
+    const double K = __dmul_rn(__ddiv_rn(q.d6, q.rhs), __hiloint2double((1023 + 2 * e) << 20, 0));
     q.K = normal && K >= 0x1p-55 && K <= 0x1p100 ? __double2float_rn(K) : nan;
     q.k = make_float4(-q.K, -q.K, kPertWindow * q.K, kPertWindow * q.K);
     q.i = i;
     q.j = k;
 }
 
-// The FP32 test of two stars against a binary: d = r^6 - L with L = K (2 m_j)^2; the
+// The FP32 test of two stars against a binary: d = r^6 - L with L = K (2 m_j 2^-e)^2; the
 // star is a perturber if d < 0, and that is certain where |d| >= w L.
 // Errors. Each component of r is a double-single difference: the high parts subtract
 // exactly when they are within a factor two of one another, so its error is at most
@@ -108,23 +124,24 @@ __device__ void load_bin(const PertArgs &P, int32_t b, Bin &q)
 // positions) compares false: undecided.
 struct Star2 {
     float2 xh, xl, yh, yl, zh, zl;   // double-single positions of two stars
-    float2 tm2;                      // (2 m)^2, NaN where the FP32 test is not to decide
+    float2 tm2;                      // (2 m 2^-e)^2, NaN where the FP32 test is not to decide
 };
 
-__device__ __forceinline__ float star_tm2(double m, float sabs, float cmax, float kmin)
+__device__ __forceinline__ float star_tm2(double m, int e, float sabs, float cmax, float kmin)
 {
     // FP64 conversions and comparisons share the narrow pipe: the mass as FP32 by bit
-    // fields (truncated, 2^-23) for |m| in [2^-34, 2^8)
-    const int hi = __double2hiint(m) & 0x7fffffff;
+    // fields (truncated, 2^-23) for |m| 2^-e in [2^-34, 2^8)
+    const int hi = (__double2hiint(m) & 0x7fffffff) - e * (1 << 20);
     const float f = __int_as_float(__funnelshift_l(__double2loint(m), hi - (896 << 20), 3));
     const float q = (2.f * f) * (2.f * f);
     const float t = 0x1p-25f * (sabs + cmax), t2 = t * t;
-    return (unsigned)(hi - ((1023 - 34) << 20)) < (unsigned)(42 << 20) && kmin * q >= (t2 * t2) * t2
+    return (unsigned)(hi - ((1023 + kMassLo) << 20)) < (unsigned)(kMassBits << 20) && kmin * q >= (t2 * t2) * t2
                ? q
                : __int_as_float(0x7fffffff);
 }
 
-__device__ __forceinline__ Star2 load_stars(const PertArgs &P, int64_t j0, int64_t j1, float cmax, float kmin)
+__device__ __forceinline__ Star2 load_stars(const PertArgs &P, int64_t j0, int64_t j1, int e, float cmax,
+                                            float kmin)
 {
     const float2 ax = __ldg(P.x2 + j0), ay = __ldg(P.x2 + P.np + j0), az = __ldg(P.x2 + 2 * P.np + j0);
     const float2 bx = __ldg(P.x2 + j1), by = __ldg(P.x2 + P.np + j1), bz = __ldg(P.x2 + 2 * P.np + j1);
@@ -136,8 +153,8 @@ __device__ __forceinline__ Star2 load_stars(const PertArgs &P, int64_t j0, int64
     t.yl = make_float2(ay.y, by.y);
     t.zh = make_float2(az.x, bz.x);
     t.zl = make_float2(az.y, bz.y);
-    t.tm2 = make_float2(star_tm2(ma, fabsf(ax.x) + fabsf(ay.x) + fabsf(az.x), cmax, kmin),
-                        star_tm2(mb, fabsf(bx.x) + fabsf(by.x) + fabsf(bz.x), cmax, kmin));
+    t.tm2 = make_float2(star_tm2(ma, e, fabsf(ax.x) + fabsf(ay.x) + fabsf(az.x), cmax, kmin),
+                        star_tm2(mb, e, fabsf(bx.x) + fabsf(by.x) + fabsf(bz.x), cmax, kmin));
     return t;
 }
 
@@ -169,9 +186,10 @@ __global__ void __launch_bounds__(kPertThreads, 4) perturbers_kernel(PertArgs P)
     __shared__ Bin bins[B];
     __shared__ unsigned bits[B][kPertSeg / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int e = mass_exp(P);
     for (int64_t b0 = (int64_t)blockIdx.x * B; b0 < P.nbin; b0 += (int64_t)gridDim.x * B) {
         __syncthreads();   // the previous binaries have been used
-        if (lane == 0 && warp < B) load_bin(P, (int32_t)(b0 + warp < P.nbin ? b0 + warp : P.nbin), bins[warp]);
+        if (lane == 0 && warp < B) load_bin(P, (int32_t)(b0 + warp < P.nbin ? b0 + warp : P.nbin), e, bins[warp]);
         __syncthreads();
         float cmax = 0.f, kmin = 0x1p100f;   // over the CTA's binaries
 #pragma unroll
@@ -192,7 +210,7 @@ __global__ void __launch_bounds__(kPertThreads, 4) perturbers_kernel(PertArgs P)
             for (int w = warp; w < words; w += 2 * kPertWarps) {
                 const int64_t ja = s0 + 32 * w + lane, jb = ja + 32 * kPertWarps;
                 const bool la = ja < P.j_hi, lb = jb < P.j_hi;
-                const Star2 t = load_stars(P, la ? ja : P.j_hi - 1, lb ? jb : P.j_hi - 1, cmax, kmin);
+                const Star2 t = load_stars(P, la ? ja : P.j_hi - 1, lb ? jb : P.j_hi - 1, e, cmax, kmin);
                 unsigned mine_a = 0, mine_b = 0;
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
