@@ -108,8 +108,12 @@ constexpr int kRing = 8;        // tiles in flight in the TMA streaming variant
 constexpr int kUnitRec = 256;
 constexpr int kUnitBytes = kUnitRec * (int)sizeof(JPair);
 constexpr int kSlots = 4;
-constexpr int kLongTiles = 12;  // variant 0: items of this many tiles go through the TMA ring (the same sums;
-                                // N = 2^20, s = 1, particles from HBM: 16.9 -> 16.5 us, no difference at 8)
+// variant 0: items of kLongTiles tiles or more go through the TMA ring where the j range is so
+// large that its records come from HBM in use (the same sums). N = 2^20, s = 1, us, ring / straight
+// loads: records from HBM 16.5 / 16.9, from L2 11.1 / 10.8; smaller ranges, which stay in L2: N =
+// 32768, s = 64 14.7 / 12.1, N = 20000, s = 64 11.6 / 10.3
+constexpr int kLongTiles = 12;
+constexpr int kColdTiles = 2048;
 constexpr int kShortTiles = 32; // shares of up to this many tiles may go by whole items (see short_items)
 
 // Resident-share variant: clusters of kShareC CTAs, CTA r holding up to
@@ -1299,7 +1303,7 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
             work_stream<2>(A, w, sm);
         else if (variant == 2)
             work_tile32(A, w, sm, git);
-        else if (variant == 0 && sm->tper < kLongTiles)
+        else if (variant == 0 && (sm->tper < kLongTiles || T < kColdTiles))
             work_stream<1>(A, w, sm);
         else
             work_stream_tma(A, w, sm, git);
