@@ -269,12 +269,32 @@ __device__ __forceinline__ void sum_lane(const float2 *src, int lane, int n, flo
     }
 }
 
+constexpr int kFewParts = 4;
+
 // Adds the n partials of each of the active particles [ib0, ib1) (slots 0 .. n - 1 of S)
 // by this CTA, in a fixed order, and writes the results.
+template <bool FEW>
 __device__ void sum_parts(const ForceArgs &A, int64_t ib0, int64_t ib1, int S, int n)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int np = (int)(ib1 - ib0);
+    if (FEW && n <= kFewParts && np <= 8) {
+        // a thread per (particle, component): no lane tree (N = 4096, s = 1 .. 16: 0.2 us, N = 24576, s =
+        // 195: 0.9 us less than the forms below)
+        if (threadIdx.x < 7 * np) {
+            const int64_t ii = ib0 + threadIdx.x / 7;
+            const int c = threadIdx.x % 7;
+            float2 v[kFewParts];
+#pragma unroll
+            for (int u = 0; u < kFewParts; ++u)
+                v[u] = u < n ? __ldcg(part2(A, ii, u, S) + c) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 1; u < kFewParts; ++u)
+                if (u < n) ds_add(v[0].x, v[0].y, v[u].x, v[u].y);
+            put_final(A, ii, c, (double)v[0].x + (double)v[0].y);
+        }
+        return;
+    }
     if (np == 1) {
         // a warp per component; lane l adds partials l, l + 32, ..., their loads issued
         // together (ten cover a partial from every CTA), then a butterfly over the lanes
@@ -331,6 +351,7 @@ __device__ void sum_parts(const ForceArgs &A, int64_t ib0, int64_t ib1, int S, i
 // Called by every thread after this CTA has written its partials of i-block bx (active
 // particles [ib0, ib1)). The CTA that completes the block's n partials (ticket n - 1)
 // adds them with two-sums and writes the FP64 results; it then re-arms the ticket.
+template <bool FEW>
 __device__ void finish_block(const ForceArgs &A, int64_t bx, int64_t ib0, int64_t ib1, int S, int n, Smem *sm)
 {
     __syncthreads();
@@ -342,7 +363,7 @@ __device__ void finish_block(const ForceArgs &A, int64_t bx, int64_t ib0, int64_
     __syncthreads();
     if (sm->last) {
         __threadfence();
-        sum_parts(A, ib0, ib1, S, n);
+        sum_parts<FEW>(A, ib0, ib1, S, n);
         if (threadIdx.x == 0) A.tickets[bx] = 0;
     }
     __syncthreads();
@@ -883,7 +904,7 @@ __device__ bool work_cols(const ForceArgs &A, int64_t s, Smem *sm)
         cols_out(A, s, ib0, lgi, n, sm->plan.part_slot, hi, lo, sm);
         if (n > 1) {
             const int64_t ib1 = ib0 + (1 << lgi);
-            finish_block(A, b, ib0, ib1 < s ? ib1 : s, P.slots, n, sm);
+            finish_block<false>(A, b, ib0, ib1 < s ? ib1 : s, P.slots, n, sm);
         }
     }
     return true;
@@ -1313,7 +1334,7 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
         }
         if (sm->split > 1) {
             const int64_t bx = qdiv(w, sm->split), i0 = bx << sm->lgi, i1 = (bx + 1) << sm->lgi;
-            finish_block(A, bx, i0, i1 < sm->s ? i1 : sm->s, sm->split, sm->split, sm);
+            finish_block<true>(A, bx, i0, i1 < sm->s ? i1 : sm->s, sm->split, sm->split, sm);
         }
     }
 }
