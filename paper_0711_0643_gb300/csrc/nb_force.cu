@@ -114,7 +114,9 @@ constexpr int kSlots = 4;
 // 32768, s = 64 14.7 / 12.1, N = 20000, s = 64 11.6 / 10.3
 constexpr int kLongTiles = 12;
 constexpr int kColdTiles = 2048;
-constexpr int kShortTiles = 32; // shares of up to this many tiles may go by whole items (see short_items)
+constexpr int kShortTiles = 32;   // shares that may go by whole items (see short_items): up to this
+constexpr int kItemTiles = 128;   //   many tiles always, up to this many where the items fill the GPU
+constexpr int kFoldTiles = kFoldPairs;   // tiles in which a thread of 256 meets kFoldPairs / 2 records
 
 // Resident-share variant: clusters of kShareC CTAs, CTA r holding up to
 // kShareRec pair records of the j range in shared memory, the active list dealt
@@ -386,13 +388,16 @@ __device__ __forceinline__ void stream_item(const ForceArgs &A, int64_t w, const
 }
 
 // The CTA's sums of particle bx, r-th of the CTA's: into the CTA's partial slot or,
-// where the CTA holds all of j (S == 1), the results.
-__device__ __forceinline__ void cta_sum_red(const Acc7 &hi, const Acc7 &lo, float2 *red)
+// where the CTA holds all of j (S == 1), the results. more: added to what is there.
+__device__ __forceinline__ void cta_sum_red(const Acc7 &hi, const Acc7 &lo, float2 *red, bool more = false)
 {
     float h, l;
     const int lane = threadIdx.x & 31;
     const int c = ds_scatter_reduce<32>(hi, lo, h, l);   // a lane holds component c
-    if ((lane & 3) == 0 && c < 7) red[c] = make_float2(h, l);
+    if ((lane & 3) == 0 && c < 7) {
+        if (more) ds_add(h, l, red[c].x, red[c].y);
+        red[c] = make_float2(h, l);
+    }
 }
 template <int R>
 __device__ __forceinline__ void cta_sum_out(const ForceArgs &A, int64_t w, Smem *sm)
@@ -416,7 +421,9 @@ __device__ __forceinline__ void cta_sum_out(const ForceArgs &A, int64_t w, Smem 
     }
 }
 
-template <int R>
+// LONG (R = 2): items of more than 64 tiles, one fold and one sum over the CTA for every 64
+// (accumulators that outlive a fold would not fit the registers).
+template <int R, bool LONG = false>
 __device__ void work_stream(const ForceArgs &A, int64_t w, Smem *sm)
 {
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -449,38 +456,47 @@ __device__ void work_stream(const ForceArgs &A, int64_t w, Smem *sm)
 #pragma unroll
     for (int r = 0; r < R; ++r) { zero(p[r]); zero(hi[r]); zero(lo[r]); }
     // two pair records per thread in flight (their loads are issued together), a fold
-    // after every kFoldPairs / 2 records (R = 2 runs on shares of up to kShortTiles
-    // tiles only, which one fold at the end covers: registers)
-    static_assert(kShortTiles / 2 <= kFoldPairs / 2, "one record per thread and two tiles");
+    // after every kFoldPairs / 2 records, i.e. 64 tiles (R = 2: at the end of them)
+    constexpr int kPart = kFoldTiles * kPT;
     int cnt = 0;
-    for (int pp = p0 + tid; pp < p1; pp += 2 * kThreads) {
-        const int pq = pp + kThreads < p1 ? pp + kThreads : pp;
-        float4 a0, a1, a2, a3, a4, b0, b1, b2, b3, b4;
-        {
-            const float4 *q = A.j.p[pp].q;
-            const float4 *w = A.j.p[pq].q;
-            a0 = __ldg(q); a1 = __ldg(q + 1); a2 = __ldg(q + 2); a3 = __ldg(q + 3); a4 = __ldg(q + 4);
-            b0 = __ldg(w); b1 = __ldg(w + 1); b2 = __ldg(w + 2); b3 = __ldg(w + 3); b4 = __ldg(w + 4);
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            pair_packed<true>(a0, a1, a2, a3, a4, ip[r], e2, p[r], 2 * pp == gi[r], 2 * pp + 1 == gi[r]);
-        if (pq != pp) {
+    bool more = false;
+    do {
+        const int pe = LONG && p1 - p0 > kPart ? p0 + kPart : p1;
+        for (int pp = p0 + tid; pp < pe; pp += 2 * kThreads) {
+            const int pq = pp + kThreads < pe ? pp + kThreads : pp;
+            float4 a0, a1, a2, a3, a4, b0, b1, b2, b3, b4;
+            {
+                const float4 *q = A.j.p[pp].q;
+                const float4 *w = A.j.p[pq].q;
+                a0 = __ldg(q); a1 = __ldg(q + 1); a2 = __ldg(q + 2); a3 = __ldg(q + 3); a4 = __ldg(q + 4);
+                b0 = __ldg(w); b1 = __ldg(w + 1); b2 = __ldg(w + 2); b3 = __ldg(w + 3); b4 = __ldg(w + 4);
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                pair_packed<true>(b0, b1, b2, b3, b4, ip[r], e2, p[r], 2 * pq == gi[r], 2 * pq + 1 == gi[r]);
-        }
-        cnt += 2;
-        if (R == 1 && cnt >= kFoldPairs / 2) {
-            cnt = 0;
-            fold(hi[0], lo[0], p[0]);
-        }
-    }
+                pair_packed<true>(a0, a1, a2, a3, a4, ip[r], e2, p[r], 2 * pp == gi[r], 2 * pp + 1 == gi[r]);
+            if (pq != pp) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        fold(hi[r], lo[r], p[r]);
-        cta_sum_red(hi[r], lo[r], &sm->red[warp][7 * r]);
-    }
+                for (int r = 0; r < R; ++r)
+                    pair_packed<true>(b0, b1, b2, b3, b4, ip[r], e2, p[r], 2 * pq == gi[r], 2 * pq + 1 == gi[r]);
+            }
+            cnt += 2;
+            if (R == 1 && cnt >= kFoldPairs / 2) {
+                cnt = 0;
+                fold(hi[0], lo[0], p[0]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            fold(hi[r], lo[r], p[r]);
+            cta_sum_red(hi[r], lo[r], &sm->red[warp][7 * r], LONG && more);
+            if (LONG) {
+                zero(hi[r]);
+                zero(lo[r]);
+            }
+        }
+        more = true;
+        p0 = pe;
+    } while (LONG && p0 < p1);
     __syncthreads();
     cta_sum_out<R>(A, w, sm);
     __syncthreads();
@@ -1225,13 +1241,20 @@ __device__ __noinline__ void share_force(const ForceArgs &A, int64_t s, Smem *sm
 }
 
 // Variants 1 and 2 where one item (two or eight particles, one share) per CTA covers the
-// block and the shares are short: such a launch is a chain of latencies, and the
-// columns' plan, ring and meeting of warps lengthen it (us under the profiler, items
-// against columns: N = 10^5, s = 2 10.4 / 17.2, s = 24 13.2 / 15.9; N = 65536, s = 20 12.4 /
-// 15.5). Longer or more items: the columns (N = 65536, s = 100 25.9 against 31.9).
+// block: short shares always, since such a launch is a chain of latencies, and the columns'
+// plan, ring and meeting of warps lengthen it (us under the profiler, items against columns: N =
+// 10^5, s = 2 10.4 / 17.2, s = 24 13.2 / 15.9; N = 65536, s = 20 12.4 / 15.5). Longer ones take as long
+// as their tiles, 9 + 0.215 t us for t of them, whatever their number; the columns as long as there
+// are particles, about 11.5 + 0.096 n us for n items of 64 to 128 tiles, whatever the share (its
+// last matrix is cut into as many units as a full one). The line is where the two meet. Items /
+// columns, us a call in a graph: N = 16385, s = 200 15.2 / 18.6, 512 23.3 / 36.0; N = 20000, s = 300 25.1 /
+// 23.0, 400 26.2 / 29.5; N = 24576, s = 257 28.8 / 23.0, 512 30.9 / 36.4; N = 49152, s = 104 19.0 / 24.5;
+// N = 32768, s = 512 38.0 / 36.0; N = 2^20, s = 20 48.1 / 54.4. More items than CTAs: the columns (N =
+// 65536, s = 65 29.9 / 22.1).
 __device__ __forceinline__ bool short_items(int variant, int64_t T, int S, int64_t items)
 {
-    return variant <= 2 && items <= gridDim.x && T <= kShortTiles * (int64_t)S;
+    return variant <= 2 && items <= gridDim.x &&
+           (T <= kShortTiles * (int64_t)S || (T <= kItemTiles * (int64_t)S && 9 * T <= (4 * items + 100) * S));
 }
 
 // SHARE: the instantiation with the resident-share variant (launched as clusters
@@ -1304,24 +1327,30 @@ __global__ void __launch_bounds__(kThreads, 2) force_mixed_kernel(ForceArgs A)
     if (blockIdx.x == 0 && tid == 0) *A.split_used = S;
     const int64_t T = A.tile_hi - A.tile_lo;
     const int lgi = variant == 1 ? 1 : (variant == 2 ? 3 : 0);
-    if (variant >= 1 && variant <= 4 && !short_items(variant, T, S, ((s + (1 << lgi) - 1) >> lgi) * S)) {
-        if (tid == 0) sm->plan = cols_plan(A, variant, s, S);
-        __syncthreads();
+    // worked out by one thread (the pair loops need the registers): the columns' plan, or the
+    // work items (i-block of 1, 2 or 8 particles, share)
+    if (tid == 0) {
+        const int64_t items = ((s + (1 << lgi) - 1) >> lgi) * S;
+        sm->items = variant < 1 || variant > 4 || short_items(variant, T, S, items) ? items : -1;
+        if (sm->items < 0) {
+            sm->plan = cols_plan(A, variant, s, S);
+        } else {
+            sm->split = S;
+            sm->lgi = lgi;
+            sm->tper = S == 1 ? T : qdiv(T + S - 1, S);
+        }
+    }
+    __syncthreads();
+    if (sm->items < 0) {
         if (blockIdx.x < sm->plan.G && !work_cols(A, s, sm) && tid == 0) atomicOr(A.status, kStTimeout);
         return;
     }
-    // work items (i-block of 1, 2 or 8 particles, share)
-    if (tid == 0) {
-        sm->split = S;
-        sm->lgi = lgi;
-        sm->tper = S == 1 ? T : qdiv(T + S - 1, S);
-        sm->items = ((s + (1 << lgi) - 1) >> lgi) * S;
-    }
-    __syncthreads();
     uint32_t git = 0;
     for (int64_t w = blockIdx.x; w < sm->items; w += gridDim.x) {
-        if (variant == 1)
+        if (variant == 1 && sm->tper <= kFoldTiles)
             work_stream<2>(A, w, sm);
+        else if (variant == 1)
+            work_stream<2, true>(A, w, sm);
         else if (variant == 2)
             work_tile32(A, w, sm, git);
         else if (variant == 0 && (sm->tper < kLongTiles || T < kColdTiles))
