@@ -266,13 +266,21 @@ nb_status nb_sync(nb_ctx *ctx);
  * split is the j-split factor at the bucket's largest size min(2^b, n); a
  * smaller block of the bucket keeps the same number of work items (i-blocks x
  * splits), so its split grows in proportion. It sets which FP32 partial sums are
- * formed; mixed variants 1 to 4 and FP64 share the work out in equal runs over
- * the GPU whatever it is.
+ * formed and, for mixed variants 0 and 5, and 1 and 2 where one wave of items covers
+ * the block, how many CTAs share the work (an item is one i-block and one share of
+ * j); variants 1 to 4 otherwise share it out in equal runs over the GPU whatever the
+ * split is. In FP64 the work is cut into equal runs too, over at most split CTAs for
+ * every i-block of the variant (1 or 32 particles): a small split leaves the rest
+ * of the GPU idle.
  * nb_get_tuning reads the table (variant[32], split[32]). */
 nb_status nb_autotune(nb_ctx *ctx);
 nb_status nb_set_tuning(nb_ctx *ctx, int32_t bucket, int32_t variant, int32_t split);
 nb_status nb_get_tuning(nb_ctx *ctx, int32_t *variant, int32_t *split);
-/* Number of force-kernel variants of the context's precision and a short name. */
+/* Number of force-kernel variants of the context's precision and a short name. The
+ * names are fixed, callers look variants up by them; they are those of the kernels
+ * the variants began as. Mixed: 0 and 5 one particle to a CTA, 1 to 4 FP32 sums over every
+ * 256th, 32nd, 8th and consecutive pair record, 6 j-records in 8-CTA clusters. FP64: 0
+ * one, 1 up to 32 particles to an i-block. */
 int32_t nb_num_variants(const nb_ctx *ctx);
 const char *nb_variant_name(const nb_ctx *ctx, int32_t variant);
 

@@ -218,13 +218,15 @@ cudaError_t launch_force_ctx(nb_ctx *c)
 // The engine's default largest block: its force phase runs on the cluster's
 // SMs only, so it takes blocks whose s N is small (2^19 pair evaluations: the
 // force phase then takes a few microseconds, below the full path's per-step
-// overhead). Above 4096 particles it is off by default: measured on this GPU, its
-// steps (~16 us at N = 16384, mostly the FP64 corrector chain and the barrier-
-// separated phases on 16 SMs) plus a launch each time a large block interrupts
-// it cost as much as the four-kernel steps (Plummer N = 16384 to t = 1: 686 vs
-// 674 ms), while at N = 1024 it saved a fifth (58 vs 75 ms). Both have become faster
-// since (N = 1024 to t = 1/4 13.2 -> 10.8 ms, N = 16384 to t = 1/16 39.0 -> 36 ms); the
-// line stays, as it also decides which FP32 partial sums a run forms.
+// overhead). Above 4096 particles it is off by default: the line was found when its
+// steps, plus a launch each time a large block interrupts it, cost as much as the
+// four-kernel steps there. Both have become faster since; Plummer models to t = 1/16
+// (N = 1024: 1/4, 2048: 1/8), ms with the engine off / for blocks of up to 16, 32, 64, 128:
+//     1024 17.1 / 15.3 13.2 12.1 11.2 (the default: 10.7)   2048 16.3 / 13.3 12.5 10.6 10.6 (10.1)
+//     4096 12.3 / 10.8 10.3 9.2 9.1 (9.1)   6000 17.3 / 14.5 14.1 13.5 12.6
+//     8192 19.5 / 19.2 17.4 17.4 16.5   12000 30.6 / 28.9 28.7 26.2 26.2   16384 35.0 / 36.6 36.3 35.8 36.5
+// So a line at 12000 would be faster by a sixth between; it also decides which FP32 partial
+// sums a run forms, and nb_set_engine moves it.
 int32_t default_engine_smax(int64_t n)
 {
     if (n > kEngDefaultMaxN) return 0;

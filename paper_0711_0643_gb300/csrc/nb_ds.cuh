@@ -109,8 +109,8 @@ __device__ __forceinline__ void ds_predict(const float2 *x2, const float2 *v2, c
     ds_predict_vals(X, V, A, K, d64, hi, lo, vel, m);
 }
 
-// Double-single helpers of the softened potential sums (the energy kernels of
-// the single-system path and of the ensemble). The two-sum steps rely on the
+// Double-single helpers of the ensemble's softened potential sums (the single-system
+// energy kernel has its own, on two pairs at a time). The two-sum steps rely on the
 // including file being compiled without multiply-add contraction.
 __device__ __forceinline__ void en_two_sum(float a, float b, float &s, float &e)
 {

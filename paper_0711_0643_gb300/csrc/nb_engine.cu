@@ -1,8 +1,8 @@
 // Small-block engine: consecutive block steps with small active blocks, each a
 // full step of Sect. 2.1 (selection by the smallest t_i + dt_i, Hermite
-// predictor for all particles, Eq. (Force) with its jerk and potential on the
-// block, corrector and Eq. (timestep) quantised to powers of two), run inside
-// one kernel by one thread-block cluster.
+// predictor for all particles, Eq. (Force) with its jerk on the block (the
+// corrector needs no potential), corrector and Eq. (timestep) quantised to powers
+// of two), run inside one kernel by one thread-block cluster.
 //
 // Why: with a few active particles a block step is a chain of dependent phases
 // whose arithmetic is small; as four kernels per step (selection, predictor,

@@ -114,7 +114,7 @@ __device__ void load_bin(const PertArgs &P, int32_t b, int e, Bin &q)
 // star is a perturber if d < 0, and that is certain where |d| >= w L.
 // Errors. Each component of r is a double-single difference: the high parts subtract
 // exactly when they are within a factor two of one another, so its error is at most
-// 2^-23 of itself plus 2^-45 X, X = the two positions' sizes. load_star admits a star
+// 2^-23 of itself plus 2^-45 X, X = the two positions' sizes. star_tm2 admits a star
 // only where 2^-45 X is below 2^-20 of the threshold distance L^(1/6), so it moves r^6
 // near the threshold by at most 6 x 2^-20 L = 2^-17.4 L; the roundings relative to r
 // add 2^-18.8 L, L itself is within 2^-21.4 of its exact value and the FP64 test rounds
@@ -283,7 +283,9 @@ cudaError_t launch_perturbers(const PertArgs &p, cudaStream_t st)
     if (p.nbin <= 0) return cudaSuccess;
     // With more binaries to a CTA each star is read less often, with fewer there are more
     // CTAs to hide a round's latency (N = 16384, us with 1, 2, 4, 8 to a CTA: 300
-    // binaries 25, 28, 37, 55; 1638 binaries 82, 70, 59, 72; 3000 140, 106, 92, 97).
+    // binaries 25, 28, 37, 55; 1638 binaries 82, 70, 59, 72; 3000 140, 106, 92, 97). The lines
+    // leave at least two CTAs of 2 or 4 binaries to each of the 152 SMs; a star's cost does
+    // not depend on N.
     if (p.nbin >= 1216) return launch_B<4>(p, st);
     if (p.nbin >= 608) return launch_B<2>(p, st);
     return launch_B<1>(p, st);

@@ -2,7 +2,7 @@
 where the first and the last star are both outside its range. Lists and counts equal to the
 FP64 oracle's with stars at the threshold, on both sides of each limit of the scaling (2^-34
 and 2^8, 2^-120 and 2^120), with the scale taken from a star that is not like the others,
-and over a j-range."""
+and over a j-range; and the numbers of binaries at which a CTA takes more of them."""
 import numpy as np
 import pytest
 
@@ -39,3 +39,10 @@ def test_range(nb, orc):  # noqa: F811
             ol, oc = orc.perturbers(m, x, pairs, gamma=gamma, nmax=100, j_lo=lo, j_hi=hi)
             np.testing.assert_array_equal(gc, oc)
             np.testing.assert_array_equal(gl, ol)
+
+
+@pytest.mark.parametrize("nbin", [607, 608, 609, 1215, 1216, 1217])
+def test_binaries_per_cta(nb, orc, nbin):  # noqa: F811
+    """One, two and four binaries to a CTA, the last CTA full and partly filled."""
+    m, x, pairs, gamma = _threshold_system(nbin, 80 + nbin, 3000)
+    _equal(nb, orc, m, x, pairs, gamma, 256)

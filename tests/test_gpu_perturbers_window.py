@@ -1,7 +1,7 @@
 """Perturber lists where the FP32 test cannot decide, and around it: stars at the
 threshold distance to within 1e-2 ... 1e-15 (relative), systems far from the origin
 (positions that need their low halves), positions and masses scaled out of the FP32
-test's range, zero masses and coincident members, for every number of binaries to a
+test's range, zero masses and coincident members, for one, two and four binaries to a
 CTA. The lists and counts are whole numbers: equal to the FP64 oracle's."""
 import numpy as np
 import pytest
@@ -53,7 +53,7 @@ def _threshold_system(nbin, seed, n_near=6000):
     return m, x, pairs, gamma
 
 
-# one binary to a CTA, two, four, eight
+# one binary to a CTA, one, two, four, four
 @pytest.mark.parametrize("nbin", [1, 100, 700, 1300, 2500])
 def test_stars_at_the_threshold(nb, orc, nbin):
     m, x, pairs, gamma = _threshold_system(nbin, 11 + nbin)
